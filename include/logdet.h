@@ -161,7 +161,8 @@ int logdet_create_device(int32_t n, const int32_t* rowptr_dev, const int32_t* co
  * w: (radius + 1)^2 doubles on the host, copied; w[0] is the diagonal (add
  * a nugget there).  The caller guarantees that Q is SPD.  The handle works
  * with every estimator, the server, plans and logdet_spmm (applied by a
- * convolution kernel, nothing n x stencil is stored); FP64 and mixed FP32
+ * convolution kernel, or in the estimators and logdet_quadform by Fourier
+ * transforms where the support is wide; nothing n x stencil is stored); FP64 and mixed FP32
  * only (EINVAL for LOGDET_MIXED_BF16VEC and LOGDET_MIXED_F32X2).  logdet_info reports n = nx * ny
  * and nnz = the entries of the implied matrix.  Errors: EINVAL (nx, ny < 1,
  * nx * ny >= 2^31, radius outside [0, 96], non-finite w), ENOTSPD

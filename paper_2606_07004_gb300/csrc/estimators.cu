@@ -261,8 +261,21 @@ int logdet_quadform(logdet_handle h, const double* x, double shift, double* out,
                             cudaMemcpyDeviceToDevice, st));
   LD_TRY(cs.alloc(ld));
   LD_TRY(fill_double(cs.p, ld, shift, st));
+  // A gridded operator with a wide support: by transforms, unless the field is
+  // not finite or their scratch does not fit (then directly, below).
+  bool by_fft = false;
   if (h->kind == 1) {
-    LD_TRY(grid_apply<double>(h, h->gtab, X.p, Y.p, ld, cs.p, st));
+    const GridFft f = grid_fft_plan<double>(h, ld);
+    if (f.pairs) {
+      DevBuf<double> tab(st);
+      int rc = tab.alloc(grid_fft_table_count<double>(f));
+      if (rc == LOGDET_OK) rc = grid_fft_table<double>(h, f, 1.0, tab.p, st);
+      if (rc == LOGDET_OK)
+        rc = grid_fft_apply<double>(h, f, tab.p, X.p, Y.p, ld, cs.p, nullptr, 0, st);
+      if (rc != LOGDET_OK && rc != LOGDET_ENOMEM) return rc;
+      by_fft = rc == LOGDET_OK;
+    }
+    if (!by_fft) LD_TRY(grid_apply<double>(h, h->gtab, X.p, Y.p, ld, cs.p, st));
   } else {
     DevBuf<double> v(st);
     const double* vals = (const double*)h->vals;
@@ -278,11 +291,15 @@ int logdet_quadform(logdet_handle h, const double* x, double shift, double* out,
   LD_TRY(part.alloc((size_t)ld * ntiles));
   LD_TRY(red.alloc(ld));
   const double* dv[1] = {X.p};
-  LD_TRY(dots_pass<double>(Y.p, dv, 1, part.p, n, ld, g.tile_rows, ntiles, g.threads, st));
-  LD_TRY(reduce_partials_fp64(part.p, ld, ntiles, red.p, st));
-  LD_CUDA(cudaMemcpyAsync(out, red.p, sizeof(double), cudaMemcpyDeviceToHost, st));
-  LD_CUDA(cudaStreamSynchronize(st));
-  return LOGDET_OK;
+  for (;;) {
+    LD_TRY(dots_pass<double>(Y.p, dv, 1, part.p, n, ld, g.tile_rows, ntiles, g.threads, st));
+    LD_TRY(reduce_partials_fp64(part.p, ld, ntiles, red.p, st));
+    LD_CUDA(cudaMemcpyAsync(out, red.p, sizeof(double), cudaMemcpyDeviceToHost, st));
+    LD_CUDA(cudaStreamSynchronize(st));
+    if (!by_fft || std::isfinite(*out)) return LOGDET_OK;
+    by_fft = false;
+    LD_TRY(grid_apply<double>(h, h->gtab, X.p, Y.p, ld, cs.p, st));
+  }
 }
 
 int logdet_orth(int32_t n, int32_t s, const double* y, int32_t ldy, double* a, int32_t lda,

@@ -200,6 +200,10 @@ int KRun<T>::init(const int* rp, const int* ci, const typename ValOf<T>::type* v
     LD_TRY(dia_err.zero());
   }
   LD_TRY(y.alloc(blk));
+  if constexpr (std::is_same<T, double>::value || std::is_same<T, float>::value) {
+    if (gfft.pairs && blk * sizeof(T) < grid_fft_own_bytes<T>(gfft, ld))
+      LD_TRY(gws.alloc(grid_fft_own_bytes<T>(gfft, ld)));
+  }
   if (!Vfull) LD_TRY(ring.alloc(blk * nring));
   LD_TRY(ks.alloc(method, b, ld, m, k, tol, rescale_limit<T>()));
   {
@@ -282,7 +286,20 @@ int KRun<T>::grid_pass1(int j) {
     return LOGDET_EINVAL;
   } else {
     using CT = typename Compute<T>::type;
-    LD_TRY(grid_apply<T>(hctx, static_cast<const CT*>(gtab), ptr(j), y.p, ld, colshift, st));
+    if (gfft.pairs) {
+      // Workspace: the block this step's update writes (dead until then); a
+      // kept basis has none after its last step.
+      void* ws = gws.p;
+      size_t bytes = gws.p ? gws.count : 0;
+      if (!ws && (!Vfull || j < m)) {
+        ws = ptr(j + 1);
+        bytes = blk * sizeof(T);
+      }
+      LD_TRY(grid_fft_apply<T>(hctx, gfft, static_cast<const T*>(gtab), ptr(j), y.p, ld, colshift, ws,
+                               bytes, st));
+    } else {
+      LD_TRY(grid_apply<T>(hctx, static_cast<const CT*>(gtab), ptr(j), y.p, ld, colshift, st));
+    }
     const T* dv[kMaxWin];
     int nd = 0;
     if (method == 0) {
@@ -602,7 +619,8 @@ struct Solve : ISolve {
   int n, s, r, b, ld, lds, m, kk;
   double lo, hi, alpha, gamma, shift;
   DevBuf<typename ValOf<T>::type> vals;
-  DevBuf<typename Compute<T>::type> gtabs;  // gridded operator: scaled table
+  DevBuf<typename Compute<T>::type> gtabs;  // gridded operator: scaled table (or transform tables)
+  GridFft gfft;                              //   the transforms' cover, if they are used
   DevBuf<float> diav;                        // FP32 values per diagonal (diagonal fast path)
   DevBuf<T> Vst, Xc;
   DevBuf<double> X64, outv, cshift;
@@ -709,7 +727,7 @@ struct Solve : ISolve {
     if (run) {
       KRun<T>& R = *run;
       KState& K = R.ks;
-      for (BufRef b : {ref(R.part), ref(R.y), ref(R.ring), ref(R.dia_err), ref(R.krun_bar),
+      for (BufRef b : {ref(R.gws), ref(R.part), ref(R.y), ref(R.ring), ref(R.dia_err), ref(R.krun_bar),
                        ref(R.krun_part2), ref(K.alpha), ref(K.beta), ref(K.H), ref(K.sig),
                        ref(K.edot), ref(K.coef), ref(K.ycoef), ref(K.dbuf), ref(K.meff),
                        ref(K.active), ref(K.status), ref(K.cnt)})
@@ -909,8 +927,17 @@ struct Solve : ISolve {
         set_error("gridded operators support FP64 and mixed FP32 blocks only");
         return LOGDET_EINVAL;
       } else {
-        LD_TRY(gtabs.alloc(grid_table_count(h)));
-        LD_TRY(grid_table<typename Compute<T>::type>(h, cscale, gtabs.p, st));
+        if constexpr (!std::is_same<T, bf16>::value) {
+          gfft = grid_fft_plan<T>(h, s ? std::min(ld, lds) : ld);
+          if (gfft.pairs) {
+            LD_TRY(gtabs.alloc(grid_fft_table_count<T>(gfft)));
+            LD_TRY(grid_fft_table<T>(h, gfft, cscale, gtabs.p, st));
+          }
+        }
+        if (!gfft.pairs) {
+          LD_TRY(gtabs.alloc(grid_table_count(h)));
+          LD_TRY(grid_table<typename Compute<T>::type>(h, cscale, gtabs.p, st));
+        }
       }
     } else {
       LD_TRY(vals.alloc(h->nnz));
@@ -936,6 +963,7 @@ struct Solve : ISolve {
       run->colshift = cshift.p;
       run->hctx = h;
       run->gtab = gtabs.p;
+      run->gfft = gfft;
       run->diavals = diav.p;
       TuneCfg tc;
       LD_TRY(layout(ld, c.method == 1, &tc));
@@ -957,7 +985,9 @@ struct Solve : ISolve {
       if constexpr (std::is_same<T, bf16>::value || std::is_same<T, f32x2>::value) {
         LD_TRY(spmm_block<T>(h->rowptr, h->colind, vals.p, n, S.p, Yt.p, lds, st, cshift.p, h));
       } else {
-        if (h->kind == 1) LD_TRY(grid_apply<T>(h, gtabs.p, S.p, Yt.p, lds, cshift.p, st));
+        if (h->kind == 1 && gfft.pairs)
+          LD_TRY(grid_fft_apply<T>(h, gfft, gtabs.p, S.p, Yt.p, lds, cshift.p, nullptr, 0, st));
+        else if (h->kind == 1) LD_TRY(grid_apply<T>(h, gtabs.p, S.p, Yt.p, lds, cshift.p, st));
         else LD_TRY(spmm_block<T>(h->rowptr, h->colind, vals.p, n, S.p, Yt.p, lds, st, cshift.p, h));
       }
       S.release();
@@ -983,6 +1013,7 @@ struct Solve : ISolve {
       run->colshift = cshift.p;
       run->hctx = h;
       run->gtab = gtabs.p;
+      run->gfft = gfft;
       run->diavals = diav.p;
       TuneCfg tc;
       LD_TRY(layout(ld, false, &tc));
@@ -995,6 +1026,7 @@ struct Solve : ISolve {
       run->colshift = cshift.p;
       run->hctx = h;
       run->gtab = gtabs.p;
+      run->gfft = gfft;
       run->diavals = diav.p;
       TuneCfg tc;
       LD_TRY(layout(lds, false, &tc));
@@ -1041,6 +1073,7 @@ struct Solve : ISolve {
     run->colshift = cshift.p;
     run->hctx = h;
     run->gtab = gtabs.p;
+    run->gfft = gfft;
     run->diavals = diav.p;
     TuneCfg tc;
     LD_TRY(layout(ld, true, &tc));

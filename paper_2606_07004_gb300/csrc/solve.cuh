@@ -16,6 +16,7 @@
 #pragma once
 
 #include "dense.cuh"
+#include "grid.cuh"
 #include "handle.cuh"
 #include "krylov.cuh"
 
@@ -92,7 +93,9 @@ struct KRun {
   const double* colshift = nullptr;  // optional [ld]: the scaled diagonal shift
   const double* colscale = nullptr;  // optional [ld]: a factor per column after the shift
   logdet_ctx* hctx = nullptr;        // matrix handle (work items of irregular matrices)
-  const void* gtab = nullptr;        // gridded operator: scaled expanded table (compute type)
+  const void* gtab = nullptr;        // gridded operator: its scaled table (compute type)
+  GridFft gfft;                      //   and the transforms' cover (gtab from grid_fft_table)
+  DevBuf<unsigned char> gws;         //   their workspace, for blocks too small to lend it
   TileGeom g{};
   TuneCfg tune{};
   int width = 0;  // columns per slice job (ld / tune.split)
@@ -111,7 +114,7 @@ struct KRun {
   cudaStream_t st;
 
   explicit KRun(cudaStream_t s)
-      : part(s), y(s), ring(s), ks(s), dia_err(s), st(s), krun_bar(s), krun_part2(s) {}
+      : gws(s), part(s), y(s), ring(s), ks(s), dia_err(s), st(s), krun_bar(s), krun_part2(s) {}
 
   // Allocate and queue the start-block norms and sigma_1 (one launch pair).
   int init(const int* rp, const int* ci, const typename ValOf<T>::type* v, int n_, long long nnz_,
