@@ -32,6 +32,13 @@ TileGeom tile_geom(int width, int vec, int threads_hint, int iters_hint, int n) 
   while (threads < 256 && threads + lcm <= 512) threads += lcm;
   if (threads > 512) threads = std::max(1, 512 / G) * G;  // very wide blocks: idle lanes accepted
   if (G > 512) threads = 512;                               // (not reached for ld <= 1024)
+  // FP64 (and double-float) blocks with fewer than two rows per SM and row
+  // group take smaller CTAs: more of them, and a shorter chain in the
+  // per-tile reductions, which add the row groups' sums one after another
+  // (64 clocks an addition in FP64).
+  while (vec == 2 && n > 0 && threads > lcm && threads % lcm == 0 &&
+         (long long)n < 2LL * sm_count() * (threads / G))
+    threads -= lcm;
   if (threads_hint > 0 && threads_hint <= 512 && threads_hint % 32 == 0 && threads_hint % G == 0)
     threads = threads_hint;
   g.threads = threads;
@@ -754,6 +761,11 @@ __global__ void __launch_bounds__(512, update_min_ctas<T, NB>())
 // values.  Which CTA arrives last does not change any value.
 // ---------------------------------------------------------------------------
 constexpr int kRedLanes = 4;  // independent accumulators per thread
+// Up to this many partials per dot the scalar steps run one warp per dot in a
+// CTA per probe (k_scalar_small): 64 x 64 grid, FP64, 256 partials: 13.4 us a
+// launch in the counter form's code, 6.6 us so; a warp per dot over the 4096
+// partials of a 2M-row block would read 128 of them one wave after another.
+constexpr int kSmallTiles = 1024;
 
 
 // Sum of the ntiles partials of (dot d, column p) by a CTA of kRedThreads
@@ -802,26 +814,65 @@ __device__ __forceinline__ int find_probe_job(const ScalarBatch& B, int gp) {
   return j;
 }
 
-// Power-of-two factor keeping the stored vectors near unit norm when sigma drifts.
-// Sigma within 2^+-(lim - 1) is well inside the limit whatever log2 rounds
-// to, so the answer 1 needs no FP64 logarithm there.
-__device__ __forceinline__ double rescale_factor(double sigma, double lim) {
-  const long long e = (long long)lim - 1;  // 2^+-e built from its bits (1 <= e <= 1000)
-  const double lo = __longlong_as_double((1023 - e) << 52), hi = __longlong_as_double((1023 + e) << 52);
-  if (sigma >= lo && sigma <= hi) return 1.0;
-  double l2 = log2(sigma);
-  if (fabs(l2) <= lim) return 1.0;
+// Power-of-two factor keeping the stored vectors near unit norm when sigma
+// drifts.  Sigma within 2^+-(lim - 1) is well inside the limit whatever log2
+// rounds to: decided on its exponent bits, without FP64 arithmetic.
+__device__ __forceinline__ double rescale_factor(double sigma, int lim) {
+  const int e = (__double2hiint(sigma) >> 20) - 1023;  // (negative sigma: a large e)
+  if (e >= 1 - lim && e < lim - 1) return 1.0;
+  const double l2 = log2(sigma);
+  if (fabs(l2) <= (double)lim) return 1.0;
   return exp2(rint(l2));
 }
 
-__device__ void scalar_init(const ScalarJob& J, int p, const double* D) {
+// 1 / sqrt(nn), the factor that normalises a stored vector of squared norm
+// nn, and *root = sqrt(nn) from it with one correction step.  An FP64
+// operation takes 64 clocks here whatever it waits for, so the scalar steps
+// form the norm, the next sigma and the pass-2 coefficients from this one
+// reciprocal root: a root and two divisions one after another made the
+// 20-probe scalar launch of a 64 x 64 grid 9.5 us of SM time.
+__device__ __forceinline__ double inv_norm(double nn, double* root) {
+  if (nn > 0.0 && nn < 1e300) {
+    const double r = rsqrt(nn);
+    const double q = nn * r;
+    *root = fma(fma(-q, q, nn), 0.5 * r, q);
+    return r;
+  }
+  *root = sqrt(nn);
+  return 1.0 / *root;
+}
+
+// The recurrences of one probe, by one warp: every lane holds the probe's
+// scalars (loaded before the reductions, whose latency hides theirs), lane 0
+// writes them, and lane t handles window vector t.  D: the reduced dots.
+struct ProbeState {
+  int act;
+  double sj, sp, beta, a;  // sigma_j, sigma_{j-1}, beta_{j-1}, pass 2's last scale
+};
+
+__device__ __forceinline__ ProbeState load_probe(const ScalarJob& J, int kind, int p) {
   const KrylovState& S = J.st;
-  const double nn = D[0];
+  const double* sg = S.sig + p * (S.m + 2);
+  ProbeState P = {0, 0.0, 0.0, 0.0, 1.0};
+  if (kind == SK_INIT) return P;
+  P.act = __ldcg(S.active + p);
+  P.sj = __ldcg(sg + J.step);
+  if (J.step >= 2) {
+    P.sp = __ldcg(sg + J.step - 1);
+    if (S.method == 0 && kind == SK_COEF) P.beta = __ldcg(S.beta + p * S.m + J.step - 2);
+  }
+  if (kind == SK_NORM || J.step >= 2) P.a = __ldcg(S.ycoef + p);
+  return P;
+}
+
+__device__ void scalar_init(const ScalarJob& J, int p, double nn) {
+  const KrylovState& S = J.st;
   const int m2 = S.m + 2;
   S.status[p] = 0;
   S.meff[p] = 0;
   if (nn > 0.0 && p < S.b) {
-    S.sig[p * m2 + 1] = 1.0 / sqrt(nn);
+    double root;
+    S.sig[p * m2 + 1] = inv_norm(nn, &root);
     S.active[p] = 1;
   } else {
     S.sig[p * m2 + 1] = 0.0;
@@ -830,100 +881,129 @@ __device__ void scalar_init(const ScalarJob& J, int p, const double* D) {
   if (S.edot) S.edot[p * m2 + 1] = nn;
 }
 
-__device__ void scalar_coef(const ScalarJob& J, int p, const double* D) {
+// Norm of u_{j+1} (step j, sigma_j = s): h = s |u_{j+1}| / a, and
+// sigma_{j+1} = s / (a h) = 1 / |u_{j+1}| (returned; 0 and the probe leaves
+// the run when it breaks down).
+__device__ __forceinline__ double scalar_norm(const ScalarJob& J, int p, int j, double s, double a,
+                                              const double* D, int ndots, int lane, int* act,
+                                              double* hout) {
   const KrylovState& S = J.st;
+  double root;
+  const double inv = inv_norm(D[0], &root);
+  double h = s * root;
+  if (a != 1.0) h = h / a;
+  const bool stop = S.method == 0 ? !(h > S.tol) /* beta_j <= tol */ : h < S.tol;
+  const double next = stop ? 0.0 : inv;
+  if (lane == 0) {
+    if (S.method == 0) S.beta[p * S.m + j - 1] = h;
+    else S.H[(size_t)p * (S.m + 1) * S.m + (size_t)(j - 1) * (S.m + 1) + j] = h;
+    if (stop) {
+      S.active[p] = 0;
+      S.status[p] |= LOGDET_ST_BREAKDOWN;
+    }
+    S.sig[p * (S.m + 2) + j + 1] = next;
+    if (S.edot) S.edot[p * (S.m + 2) + j + 1] = ndots > 1 ? D[1] : 0.0;
+  }
+  if (stop) *act = 0;
+  *hout = h;
+  return next;
+}
+
+// Pass-2 coefficient of u_{j-1} in Lanczos: a beta sigma_{j-1} / sigma_j, with
+// sigma_{j-1} / sigma_j = a_{j-1} beta.
+__device__ __forceinline__ double lanczos_back_coef(double a, double a_prev, double beta) {
+  return a * a_prev * (beta * beta);
+}
+
+__device__ void scalar_recur(const ScalarJob& J, int kind, int p, ProbeState P, const double* D) {
+  const KrylovState& S = J.st;
+  const int lane = threadIdx.x & 31;
   const int j = J.step;
-  const int m2 = S.m + 2;
-  const double* sg = S.sig + p * m2;
-  double* coef = S.coef;
-  if (!S.active[p]) {
-    S.ycoef[p] = 0.0;
-    for (int t = 0; t < kMaxWin; ++t) coef[t * S.ld + p] = 0.0;
+  if (kind == SK_INIT) {
+    if (lane == 0) scalar_init(J, p, D[0]);
     return;
   }
-  S.meff[p] = j;
-  const double sj = sg[j];
-  const double a = rescale_factor(sj, S.rescale_lim);
+  double h;
+  if (kind == SK_NORM) {
+    if (P.act) scalar_norm(J, p, j, P.sj, P.a, D, J.ndots, lane, &P.act, &h);
+    return;
+  }
+  if (J.nndots && P.act) {
+    // the norm of the step before, left for this launch
+    P.sj = scalar_norm(J, p, j - 1, P.sp, P.a, D, J.nndots, lane, &P.act, &h);
+    P.beta = h;
+  }
+  D += J.nndots;
+  double* coef = S.coef;
+  if (!P.act) {
+    if (lane == 0) S.ycoef[p] = 0.0;
+    if (lane < kMaxWin) coef[lane * S.ld + p] = 0.0;
+    return;
+  }
+  const double a = rescale_factor(P.sj, S.rescale_lim);
   if (S.method == 0) {
-    const double al = sj * sj * D[0];
-    S.alpha[p * S.m + j - 1] = al;
-    if (j >= 2) {
-      coef[0 * S.ld + p] = a * S.beta[p * S.m + j - 2] * sg[j - 1] / sj;
-      coef[1 * S.ld + p] = a * al;
-    } else {
-      coef[0 * S.ld + p] = a * al;
+    const double al = P.sj * P.sj * D[0];
+    if (lane == 0) {
+      S.alpha[p * S.m + j - 1] = al;
+      if (j >= 2) {
+        coef[0 * S.ld + p] = lanczos_back_coef(a, P.a, P.beta);
+        coef[1 * S.ld + p] = a * al;
+      } else {
+        coef[0 * S.ld + p] = a * al;
+      }
     }
-  } else {
-    double* Hc = S.H + (size_t)p * (S.m + 1) * S.m + (size_t)(j - 1) * (S.m + 1);
-    for (int t = 0; t < J.ndots; ++t) {
-      const int i = J.win_lo + t;
-      Hc[i - 1] = sg[i] * sj * D[t];
-      coef[t * S.ld + p] = a * sg[i] * sg[i] * D[t];
-    }
+  } else if (lane < J.ndots) {
+    const int i = J.win_lo + lane;
+    const double si = i == j ? P.sj : __ldcg(S.sig + p * (S.m + 2) + i);
+    S.H[(size_t)p * (S.m + 1) * S.m + (size_t)(j - 1) * (S.m + 1) + i - 1] = si * P.sj * D[lane];
+    coef[lane * S.ld + p] = a * si * si * D[lane];
   }
-  S.ycoef[p] = a;
-}
-
-__device__ void scalar_norm(const ScalarJob& J, int p, const double* D) {
-  const KrylovState& S = J.st;
-  if (!S.active[p]) return;
-  const double nn = D[0];
-  const double ee = J.ndots > 1 ? D[1] : 0.0;
-  const int j = J.step;
-  const int m2 = S.m + 2;
-  double* sg = S.sig + p * m2;
-  const double a = S.ycoef[p];
-  const double h = sg[j] * sqrt(nn) / a;
-  bool stop;
-  if (S.method == 0) {
-    S.beta[p * S.m + j - 1] = h;
-    stop = !(h > S.tol);          // beta_j <= tol
-  } else {
-    S.H[(size_t)p * (S.m + 1) * S.m + (size_t)(j - 1) * (S.m + 1) + j] = h;
-    stop = h < S.tol;
-  }
-  if (stop) {
-    S.active[p] = 0;
-    S.status[p] |= LOGDET_ST_BREAKDOWN;
-    sg[j + 1] = 0.0;
-  } else {
-    sg[j + 1] = sg[j] / (a * h);
-  }
-  if (S.edot) S.edot[p * m2 + j + 1] = ee;
-}
-
-// Dot d of probe p of a scalar job by one CTA: reduce its partials; the last
-// of the probe's dots to arrive runs the recurrence.
-template <typename Acc, typename PartT>
-__device__ void scalar_item(const ScalarJob& J, int kind, int p, int d, Acc* sh) {
-  const KrylovState& S = J.st;
-  const double v = reduce_partials<Acc, PartT>(static_cast<const PartT*>(J.part), S.ld, J.ntiles,
-                                               d, p, sh);
-  if (threadIdx.x == 0) {
-    S.dbuf[d * S.ld + p] = v;
-    __threadfence();
-    const unsigned ticket = atomicAdd(S.cnt + p, 1u);
-    if (ticket == (unsigned)(J.ndots - 1)) {
-      S.cnt[p] = 0;
-      __threadfence();
-      double D[kMaxWin];
-      for (int t = 0; t < J.ndots; ++t) D[t] = __ldcg(S.dbuf + t * S.ld + p);
-      if (kind == SK_INIT) scalar_init(J, p, D);
-      else if (kind == SK_COEF) scalar_coef(J, p, D);
-      else scalar_norm(J, p, D);
-    }
+  if (lane == 0) {
+    S.meff[p] = j;
+    S.ycoef[p] = a;
   }
 }
 
+// Dot t of a scalar job: the pending norm dots first, then its own.
+struct DotOf {
+  const void* part;
+  int ntiles, d;
+};
+__device__ __forceinline__ DotOf dot_of(const ScalarJob& J, int t) {
+  if (t < J.nndots) return {J.npart, J.nntiles, t};
+  return {J.part, J.ntiles, t - J.nndots};
+}
+
+// Large blocks: dot d of probe p by one CTA; the last of the probe's dots to
+// arrive runs the recurrences.
 template <typename Acc, typename PartT>
 __device__ void scalar_body(const ScalarBatch& B, int kind, Acc* sh) {
+  __shared__ int s_last;
+  __shared__ double D[kMaxWin + 2];
   const int gp = blockIdx.x;
-  const int d = blockIdx.y;
+  const int t = blockIdx.y;
   const int jb = find_probe_job(B, gp);
   const ScalarJob& J = B.jobs[jb];
+  const KrylovState& S = J.st;
   const int p = gp - B.probe_start[jb];
-  if (d >= J.ndots) return;
-  scalar_item<Acc, PartT>(J, kind, p, d, sh);
+  const int total = J.ndots + J.nndots;
+  if (t >= total) return;
+  const DotOf w = dot_of(J, t);
+  const double v =
+      reduce_partials<Acc, PartT>(static_cast<const PartT*>(w.part), S.ld, w.ntiles, w.d, p, sh);
+  if (threadIdx.x == 0) {
+    S.dbuf[t * S.ld + p] = v;
+    __threadfence();
+    s_last = atomicAdd(S.cnt + p, 1u) == (unsigned)(total - 1);
+  }
+  __syncthreads();
+  if (!s_last || threadIdx.x >= 32) return;
+  const ProbeState P = load_probe(J, kind, p);
+  if (threadIdx.x == 0) S.cnt[p] = 0;
+  __threadfence();
+  if (threadIdx.x < total) D[threadIdx.x] = __ldcg(S.dbuf + threadIdx.x * S.ld + p);
+  __syncwarp();
+  scalar_recur(J, kind, p, P, D);
 }
 
 __global__ void __launch_bounds__(kRedThreads) k_scalar(const __grid_constant__ ScalarBatch B,
@@ -933,6 +1013,133 @@ __global__ void __launch_bounds__(kRedThreads) k_scalar(const __grid_constant__ 
   pdl_entry();
   if (f32) scalar_body<AccF, float2>(B, kind, shf);
   else scalar_body<AccD, double>(B, kind, shd);
+}
+
+// One warp's copy of reduce_partials for (dot d, column p): lane L stands in
+// for the reduction threads L, L + 32, ..., L + 224, each accumulating the
+// same tiles into the same lanes, then the same tree (the first three levels
+// within a lane, the last five by shuffles), so the value is bit-identical
+// to the 256-thread reduction of k_scalar.  Partials are read through L2.
+template <typename Acc>
+__device__ __forceinline__ Acc shfl_down_acc(const Acc& a, int w);
+template <>
+__device__ __forceinline__ AccD shfl_down_acc<AccD>(const AccD& a, int w) {
+  AccD o;
+  o.s = __shfl_down_sync(0xffffffffu, a.s, w);
+  return o;
+}
+template <>
+__device__ __forceinline__ AccF shfl_down_acc<AccF>(const AccF& a, int w) {
+  AccF o;
+  o.s = __shfl_down_sync(0xffffffffu, a.s, w);
+  o.e = __shfl_down_sync(0xffffffffu, a.e, w);
+  return o;
+}
+
+template <typename Acc, typename PartT>
+__device__ double warp_reduce_partials(const PartT* part, int ld, int ntiles, int d, int p) {
+  static_assert(kRedThreads == 256, "the warp copy stands in for 8 threads per lane");
+  const int L = threadIdx.x & 31;
+  const PartT* src = part + ((size_t)d * ld + p) * ntiles;
+  if (ntiles <= kRedThreads) {
+    // At most one partial per reduction thread: eight loads in flight, then
+    // the tree, in a third of the instructions of the general form below
+    // (which a lone warp issues at about 20 clocks each).  Slots past ntiles
+    // hold +0, which changes no sum.
+    PartT x[8];
+    Acc v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (L + 32 * k < ntiles) x[k] = __ldcg(src + L + 32 * k);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      v[k].zero();
+      if (L + 32 * k < ntiles) get_part(x + k, v[k]);
+    }
+#pragma unroll
+    for (int w = 4; w >= 1; w >>= 1)
+#pragma unroll
+      for (int k = 0; k < w; ++k)
+        if (32 * w < ntiles) v[k].add(v[k + w]);
+#pragma unroll
+    for (int w = 16; w >= 1; w >>= 1) {
+      const Acc o = shfl_down_acc(v[0], w);
+      if (L < w) v[0].add(o);
+    }
+    return __shfl_sync(0xffffffffu, v[0].value(), 0);
+  }
+  // Slots (reduction threads) that hold data: the others stay +0, and the
+  // additions of +0 that the 256-thread tree makes leave a value unchanged
+  // (accumulators start at +0 and never become -0), so they are skipped.
+  int nz = min(ntiles, kRedThreads);
+  Acc v[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int t = L + 32 * k;
+    Acc a[kRedLanes];
+#pragma unroll
+    for (int l = 0; l < kRedLanes; ++l) a[l].zero();
+    if (t < nz) {
+      for (int base = t; base < ntiles; base += kRedThreads * kRedLanes) {
+#pragma unroll
+        for (int l = 0; l < kRedLanes; ++l) {
+          const int i = base + l * kRedThreads;
+          if (i < ntiles) {
+            const PartT x = __ldcg(src + i);
+            Acc o;
+            get_part(&x, o);
+            a[l].add(o);
+          }
+        }
+      }
+#pragma unroll
+      for (int l = 1; l < kRedLanes; ++l)
+        if (l * kRedThreads < ntiles) a[0].add(a[l]);  // (the others are +0 too)
+    }
+    v[k] = a[0];
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k)                       // w = 128
+    if (L + 32 * k + 128 < nz) v[k].add(v[k + 4]);
+  nz = min(nz, 128);
+#pragma unroll
+  for (int k = 0; k < 2; ++k)                       // w = 64
+    if (L + 32 * k + 64 < nz) v[k].add(v[k + 2]);
+  nz = min(nz, 64);
+  if (L + 32 < nz) v[0].add(v[1]);                  // w = 32
+  nz = min(nz, 32);
+#pragma unroll
+  for (int w = 16; w >= 1; w >>= 1) {               // w = 16 .. 1
+    const Acc o = shfl_down_acc(v[0], w);
+    if (L + w < nz) v[0].add(o);                    // (implies L < w: nz <= 2w here)
+    nz = min(nz, w);
+  }
+  return __shfl_sync(0xffffffffu, v[0].value(), 0);
+}
+
+// Small blocks (few partials per dot): one CTA per probe, a warp per dot, so
+// no counter and no second trip through memory stand between the reductions
+// and the recurrences.  The values are those of k_scalar, bit for bit.
+__global__ void __launch_bounds__(32 * (kMaxWin + 2)) k_scalar_small(
+    const __grid_constant__ ScalarBatch B, int kind, int f32) {
+  __shared__ double D[kMaxWin + 2];
+  pdl_entry();
+  const int gp = blockIdx.x;
+  const int jb = find_probe_job(B, gp);
+  const ScalarJob& J = B.jobs[jb];
+  const int p = gp - B.probe_start[jb];
+  const int t = threadIdx.x >> 5;
+  ProbeState P;
+  if (t == 0) P = load_probe(J, kind, p);
+  if (t < J.ndots + J.nndots) {
+    const DotOf w = dot_of(J, t);
+    const double v =
+        f32 ? warp_reduce_partials<AccF>(static_cast<const float2*>(w.part), J.st.ld, w.ntiles, w.d, p)
+            : warp_reduce_partials<AccD>(static_cast<const double*>(w.part), J.st.ld, w.ntiles, w.d, p);
+    if ((threadIdx.x & 31) == 0) D[t] = v;
+  }
+  __syncthreads();
+  if (t == 0) scalar_recur(J, kind, p, P, D);
 }
 
 // ---------------------------------------------------------------------------
@@ -990,80 +1197,6 @@ __device__ __forceinline__ T* run_ptr(const PersistRun<T>& P, int i) {
   return P.ring + (size_t)((i - 2) % P.nring) * P.blk;
 }
 
-// One warp's copy of reduce_partials for (dot d, column p): lane L stands in
-// for the reduction threads L, L + 32, ..., L + 224, each accumulating the
-// same tiles into the same lanes, then the same tree (the first three levels
-// within a lane, the last five by shuffles), so the value is bit-identical
-// to the 256-thread reduction of k_scalar.  Partials are read through L2.
-template <typename Acc>
-__device__ __forceinline__ Acc shfl_down_acc(const Acc& a, int w);
-template <>
-__device__ __forceinline__ AccD shfl_down_acc<AccD>(const AccD& a, int w) {
-  AccD o;
-  o.s = __shfl_down_sync(0xffffffffu, a.s, w);
-  return o;
-}
-template <>
-__device__ __forceinline__ AccF shfl_down_acc<AccF>(const AccF& a, int w) {
-  AccF o;
-  o.s = __shfl_down_sync(0xffffffffu, a.s, w);
-  o.e = __shfl_down_sync(0xffffffffu, a.e, w);
-  return o;
-}
-
-template <typename Acc, typename PartT>
-__device__ double warp_reduce_partials(const PartT* part, int ld, int ntiles, int d, int p) {
-  static_assert(kRedThreads == 256, "the warp copy stands in for 8 threads per lane");
-  const int L = threadIdx.x & 31;
-  const PartT* src = part + ((size_t)d * ld + p) * ntiles;
-  // Slots (reduction threads) that hold data: the others stay +0, and the
-  // additions of +0 that the 256-thread tree makes leave a value unchanged
-  // (accumulators start at +0 and never become -0), so they are skipped.
-  int nz = min(ntiles, kRedThreads);
-  Acc v[8];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const int t = L + 32 * k;
-    Acc a[kRedLanes];
-#pragma unroll
-    for (int l = 0; l < kRedLanes; ++l) a[l].zero();
-    if (t < nz) {
-      for (int base = t; base < ntiles; base += kRedThreads * kRedLanes) {
-#pragma unroll
-        for (int l = 0; l < kRedLanes; ++l) {
-          const int i = base + l * kRedThreads;
-          if (i < ntiles) {
-            const PartT x = __ldcg(src + i);
-            Acc o;
-            get_part(&x, o);
-            a[l].add(o);
-          }
-        }
-      }
-#pragma unroll
-      for (int l = 1; l < kRedLanes; ++l) a[0].add(a[l]);
-    }
-    v[k] = a[0];
-  }
-#pragma unroll
-  for (int k = 0; k < 4; ++k)                       // w = 128
-    if (L + 32 * k + 128 < nz) v[k].add(v[k + 4]);
-  nz = min(nz, 128);
-#pragma unroll
-  for (int k = 0; k < 2; ++k)                       // w = 64
-    if (L + 32 * k + 64 < nz) v[k].add(v[k + 2]);
-  nz = min(nz, 64);
-  if (L + 32 < nz) v[0].add(v[1]);                  // w = 32
-  nz = min(nz, 32);
-#pragma unroll
-  for (int w = 16; w >= 1; w >>= 1) {               // w = 16 .. 1
-    const Acc o = shfl_down_acc(v[0], w);
-    if (L + w < nz) v[0].add(o);                    // (implies L < w: nz <= 2w here)
-    nz = min(nz, w);
-  }
-  return __shfl_sync(0xffffffffu, v[0].value(), 0);
-}
-
 // Shared-memory state of a persistent run: every CTA keeps the per-probe
 // scalars the recurrences read (recent sigmas, the last beta, the active
 // flags) and the pass-2 coefficients, and runs the recurrences itself, so a
@@ -1098,7 +1231,7 @@ __device__ __forceinline__ void run_coef(const KrylovState& S, RunShared& R, int
     const double al = sj * sj * R.D[0][p];
     if (writer) S.alpha[p * S.m + j - 1] = al;
     if (j >= 2) {
-      R.cf[0 * ld + p] = a * R.beta_prev[p] * sg[(j - 1) % kSgRing] / sj;
+      R.cf[0 * ld + p] = lanczos_back_coef(a, R.yc[p], R.beta_prev[p]);
       R.cf[1 * ld + p] = a * al;
     } else {
       R.cf[0 * ld + p] = a * al;
@@ -1124,7 +1257,10 @@ __device__ __forceinline__ void run_norm(const KrylovState& S, RunShared& R, int
   const int m2 = S.m + 2;
   const double a = R.yc[p];
   const double sgj = R.sg[p][j % kSgRing];
-  const double h = sgj * sqrt(nn) / a;
+  double root;
+  const double inv = inv_norm(nn, &root);
+  double h = sgj * root;
+  if (a != 1.0) h = h / a;
   bool stop;
   if (S.method == 0) {
     R.beta_prev[p] = h;
@@ -1143,7 +1279,7 @@ __device__ __forceinline__ void run_norm(const KrylovState& S, RunShared& R, int
     }
     next = 0.0;
   } else {
-    next = sgj / (a * h);
+    next = inv;
   }
   R.sg[p][(j + 1) % kSgRing] = next;
   if (writer) {
@@ -1271,7 +1407,7 @@ static int persistent_grid(K kernel, int threads, size_t smem, int total_tiles) 
 // Launch with programmatic stream serialization (see pdl_entry).
 template <typename... KArgs, typename... Args>
 static void launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                       Args... args) {
+                       const Args&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -1309,9 +1445,13 @@ int launch_spmm(const SpmmBatch<T>& b, int threads, cudaStream_t s) {
   {                                                                           \
     auto kern = items ? spmm_kernel<T, ND, true>() : spmm_kernel<T, ND, false>(); \
     int grid = persistent_grid(kern, threads, smem, b.total_tiles);           \
-    launch_pdl(kern, dim3(grid), dim3(threads), smem, s, b);                  \
+    if (b.total_tiles <= kSmallTiles) launch_pdl(kern, dim3(grid), dim3(threads), smem, s, b); \
+    else kern<<<grid, threads, smem, s>>>(b);                                 \
     break;                                                                    \
   }
+  // A large pass 1 is launched without the overlap: it follows the update
+  // pass, and CTAs resident beside that pass's ran 4 % slower (128^3 FP64,
+  // window 4: 211.4 ms a solve against 206.0).
   do {
     if (nd == 0) LD_SPMM_CASE(0)
     if (nd == 1) LD_SPMM_CASE(1)
@@ -1425,10 +1565,16 @@ template int launch_krylov_run<float>(const PersistRun<float>&, int, int, int, c
 static int total_probes(const ScalarBatch& b) { return b.probe_start[b.njobs]; }
 
 static int launch_scalar(const ScalarBatch& b, int kind, cudaStream_t s) {
-  int nd = 1, f32 = b.jobs[0].part_f32;
-  for (int j = 0; j < b.njobs; ++j) nd = std::max(nd, b.jobs[j].ndots);
+  int nd = 1, tiles = 0, f32 = b.jobs[0].part_f32;
+  for (int j = 0; j < b.njobs; ++j) {
+    nd = std::max(nd, b.jobs[j].ndots + b.jobs[j].nndots);
+    tiles = std::max(tiles, std::max(b.jobs[j].ntiles, b.jobs[j].nntiles));
+  }
   ProfScope prof(KC_SCALAR, s);
-  launch_pdl(k_scalar, dim3(total_probes(b), nd), dim3(kRedThreads), 0, s, b, kind, f32);
+  if (tiles <= kSmallTiles)
+    launch_pdl(k_scalar_small, dim3(total_probes(b)), dim3(32 * nd), 0, s, b, kind, f32);
+  else
+    launch_pdl(k_scalar, dim3(total_probes(b), nd), dim3(kRedThreads), 0, s, b, kind, f32);
   LD_CHECK_LAUNCH();
   return LOGDET_OK;
 }

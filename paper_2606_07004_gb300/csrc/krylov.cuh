@@ -117,7 +117,7 @@ struct KrylovState {
   int method;        // 0 = Lanczos (3-term), 1 = IOP window k
   int b, ld, m, k;   // probes, leading dim, max steps, window
   double tol;
-  double rescale_lim;  // |log2 sigma| beyond which a power-of-two rescale is applied
+  int rescale_lim;  // |log2 sigma| beyond which a power-of-two rescale is applied
   double* alpha;     // Lanczos: [p*m + j-1]
   double* beta;      // Lanczos: [p*m + j-1]  (beta_j, j = 1..m-1)
   double* H;         // IOP: [p*(m+1)*m + (j-1)*(m+1) + (i-1)]  column-major H(i,j)
@@ -128,7 +128,7 @@ struct KrylovState {
   int* meff;         // [p] completed steps
   int* active;       // [p]
   uint32_t* status;  // [p] status bits
-  double* dbuf;      // [kMaxWin][ld] reduced dots of the current scalar step
+  double* dbuf;      // [kMaxWin + 2][ld] reduced dots of the current scalar step
   unsigned* cnt;     // [ld] arrival counters (zero between launches)
 };
 
@@ -139,6 +139,12 @@ struct ScalarJob {
   int ntiles;
   int step;           // j (1-based)
   int ndots;          // number of dots in part
+  // SK_COEF: pass-2 partials of the step before, whose norm this launch runs
+  // first (nndots == 0: it already ran).  Pass 1 needs no scalars (its input
+  // is not normalised), so nothing waits for the norm until then, and a step
+  // takes three launches instead of four.
+  const void* npart;
+  int nntiles, nndots;
   int win_lo;         // first window index i (1-based) for IOP / Lanczos
   int last;           // 1 = last step (no pass 2 follows)
 };

@@ -93,7 +93,7 @@ int validate_cfg(const logdet_ctx* h, const SolveCfg& c) {
 // ---------------------------------------------------------------------------
 // KState / KRun
 // ---------------------------------------------------------------------------
-int KState::alloc(int method, int b, int ld, int m, int k, double tol, double rescale_lim) {
+int KState::alloc(int method, int b, int ld, int m, int k, double tol, int rescale_lim) {
   if (method == 0) {
     LD_TRY(alpha.alloc((size_t)ld * m));
     LD_TRY(beta.alloc((size_t)ld * m));
@@ -107,7 +107,7 @@ int KState::alloc(int method, int b, int ld, int m, int k, double tol, double re
   LD_TRY(edot.alloc((size_t)ld * (m + 2)));
   LD_TRY(coef.alloc((size_t)kMaxWin * ld));
   LD_TRY(ycoef.alloc(ld));
-  LD_TRY(dbuf.alloc((size_t)kMaxWin * ld));
+  LD_TRY(dbuf.alloc((size_t)(kMaxWin + 2) * ld));
   LD_TRY(meff.alloc(ld));
   LD_TRY(active.alloc(ld));
   LD_TRY(status.alloc(ld));
@@ -195,6 +195,11 @@ int KRun<T>::init(const int* rp, const int* ci, const typename ValOf<T>::type* v
   ndmax = std::max(win, 2);
   nring = win + 1;
   LD_TRY(part.alloc((size_t)ndmax * ld * std::max(ntiles, nslots)));
+  // Lanczos leaves the second dot's place in part free for the norms; a
+  // window run has a buffer of its own, up to a size the memory estimate
+  // covers (beyond it the norm runs right after its pass, from part).
+  if (method != 0 && (size_t)2 * ld * ntiles * sizeof(Part) <= kNormPartMax)
+    LD_TRY(npart.alloc((size_t)2 * ld * ntiles));
   if (diavals) {
     LD_TRY(dia_err.alloc(1));
     LD_TRY(dia_err.zero());
@@ -320,7 +325,7 @@ void KRun<T>::upd_jobs(int j, std::vector<UpdJob<T>>& out) const {
     U.coef = ks.coef.p;
     U.ycoef = ks.ycoef.p;
     U.extra = track_e ? X0 : nullptr;
-    U.part = part.p;
+    U.part = norm_part();
     U.n = n;
     U.ld = ld;
     U.col_off = q * width;
@@ -359,6 +364,11 @@ ScalarJob KRun<T>::scalar_job(int j, int ndots, bool spmm_pass) const {
   sj.ndots = ndots;
   sj.win_lo = j >= 1 ? win_lo(j) : 1;
   sj.last = j == m;
+  if (spmm_pass && late_norm() && j > 1) {
+    sj.npart = norm_part();
+    sj.nntiles = ntiles;
+    sj.nndots = track_e ? 2 : 1;
+  }
   return sj;
 }
 
@@ -397,7 +407,7 @@ int KRun<T>::issue_rest_persistent() {
     P.sj = sj[0];
     P.uj = uj[0];
     P.uj.part = krun_part2.p;  // pass-2 partials apart from pass 1's
-    P.cj = scalar_job(j, 1, true);
+    P.cj = scalar_job(j, 1, true);  // (from step 1: no pending norm)
     P.X0 = X0;
     P.ring = ring.p;
     P.Vfull = Vfull;
@@ -727,7 +737,7 @@ struct Solve : ISolve {
     if (run) {
       KRun<T>& R = *run;
       KState& K = R.ks;
-      for (BufRef b : {ref(R.gws), ref(R.part), ref(R.y), ref(R.ring), ref(R.dia_err), ref(R.krun_bar),
+      for (BufRef b : {ref(R.gws), ref(R.part), ref(R.npart), ref(R.y), ref(R.ring), ref(R.dia_err), ref(R.krun_bar),
                        ref(R.krun_part2), ref(K.alpha), ref(K.beta), ref(K.H), ref(K.sig),
                        ref(K.edot), ref(K.coef), ref(K.ycoef), ref(K.dbuf), ref(K.meff),
                        ref(K.active), ref(K.status), ref(K.cnt)})
@@ -1147,6 +1157,7 @@ struct Solve : ISolve {
     if (!run->has_pass2(j)) return false;
     auto& v = *static_cast<std::vector<UpdJob<T>>*>(vec);
     run->upd_jobs(j, v);
+    if (run->late_norm()) return true;
     norm.push_back(run->scalar_job(j, run->track_e ? 2 : 1));
     widths.push_back(run->ld);
     return true;
@@ -1451,6 +1462,7 @@ struct GroupSolve : ISolve {
     if (!w->has_pass2(j)) return false;
     auto& v = *static_cast<std::vector<UpdJob<T>>*>(vec);
     w->upd_jobs(j, v);
+    if (w->late_norm()) return true;
     norm.push_back(w->scalar_job(j, w->track_e ? 2 : 1));
     widths.push_back(w->ld);
     return true;
@@ -1572,8 +1584,9 @@ int solve_blocking(logdet_ctx* h, const SolveCfg& c, cudaStream_t st, SolveOut& 
   return sv->assemble(o);
 }
 
-// One Krylov step of a solve whose blocks hold T: pass 1, its scalar
-// kernel, then (where the step has one) pass 2 and its scalar kernel.
+// One Krylov step of a solve whose blocks hold T: pass 1, its scalar kernel,
+// then (where the step has one) pass 2 and, unless the next step's scalar
+// kernel takes its norm too, another scalar kernel.
 template <typename T>
 static int issue_step_t(ISolve* sv, int th, cudaStream_t st) {
   thread_local std::vector<SpmmJob<T>> sp;
@@ -1587,7 +1600,7 @@ static int issue_step_t(ISolve* sv, int th, cudaStream_t st) {
   sj.clear(); widths.clear();
   if (sv->add_pass2(&up, sj, widths)) {
     LD_TRY(launch_update_jobs<T>(up, th, st));
-    LD_TRY(launch_scalar_jobs(sj, widths, SK_NORM, st));
+    if (!sj.empty()) LD_TRY(launch_scalar_jobs(sj, widths, SK_NORM, st));
   }
   return LOGDET_OK;
 }

@@ -65,14 +65,14 @@ struct KState {
   explicit KState(cudaStream_t s)
       : alpha(s), beta(s), H(s), sig(s), edot(s), coef(s), ycoef(s), dbuf(s), meff(s), active(s),
         status(s), cnt(s) {}
-  int alloc(int method, int b, int ld, int m, int k, double tol, double rescale_lim);
+  int alloc(int method, int b, int ld, int m, int k, double tol, int rescale_lim);
 };
 
-template <typename T> constexpr double rescale_limit();
-template <> constexpr double rescale_limit<double>() { return 200.0; }
-template <> constexpr double rescale_limit<float>() { return 20.0; }
-template <> constexpr double rescale_limit<bf16>() { return 20.0; }
-template <> constexpr double rescale_limit<f32x2>() { return 20.0; }
+template <typename T> constexpr int rescale_limit();
+template <> constexpr int rescale_limit<double>() { return 200; }
+template <> constexpr int rescale_limit<float>() { return 20; }
+template <> constexpr int rescale_limit<bf16>() { return 20; }
+template <> constexpr int rescale_limit<f32x2>() { return 20; }
 
 // One Krylov run over a block X0 (n x ld, b live columns): method 0 is
 // three-term Lanczos, method 1 IOP with window k.  With Vfull the basis is
@@ -103,7 +103,7 @@ struct KRun {
   const int4* items = nullptr;  // SpMM work items (nullptr: uniform tiles)
   int nslots = 0;               // SpMM partial slots per column (ntiles or the item count)
   size_t blk = 0;
-  DevBuf<Part> part;
+  DevBuf<Part> part, npart;
   DevBuf<T> y, ring;
   KState ks;
   const float* diavals = nullptr;  // FP32 values per row and diagonal: the line-sweep path
@@ -114,7 +114,7 @@ struct KRun {
   cudaStream_t st;
 
   explicit KRun(cudaStream_t s)
-      : gws(s), part(s), y(s), ring(s), ks(s), dia_err(s), st(s), krun_bar(s), krun_part2(s) {}
+      : gws(s), part(s), npart(s), y(s), ring(s), ks(s), dia_err(s), st(s), krun_bar(s), krun_part2(s) {}
 
   // Allocate and queue the start-block norms and sigma_1 (one launch pair).
   int init(const int* rp, const int* ci, const typename ValOf<T>::type* v, int n_, long long nnz_,
@@ -127,6 +127,12 @@ struct KRun {
   bool finished() const { return done_steps >= m; }
   bool has_pass2(int j) const { return j < m; }
   int pass1_dots(int j) const { return method == 0 ? 1 : j - win_lo(j) + 1; }
+  // Where pass 2 leaves its partials, and whether they keep until the next
+  // step's scalar launch (pass 1's partials do not overwrite them).
+  Part* norm_part() const {
+    return method == 0 ? part.p + (size_t)ld * std::max(ntiles, nslots) : npart.p ? npart.p : part.p;
+  }
+  bool late_norm() const { return method == 0 || npart.p; }
   // Step j's jobs, one per column slice.
   int spmm_jobs(int j, std::vector<SpmmJob<T>>& out) const;
   // Gridded operator: step j's pass 1 (y = Q~ u_j and the window dots),
@@ -145,6 +151,9 @@ struct KRun {
   DevBuf<unsigned> krun_bar;
   DevBuf<Part> krun_part2;  // persistent run: pass-2 partials
 };
+
+// Largest buffer of norm partials a window run keeps apart (see norm_part).
+constexpr size_t kNormPartMax = (size_t)4 << 20;
 
 // Blocks up to this size (bytes of one n x ld block) may run their Krylov
 // steps as one persistent launch in the blocking and graph-plan paths.
