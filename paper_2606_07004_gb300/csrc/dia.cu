@@ -27,6 +27,7 @@
 // their compensated partial sums.
 #include "dia.cuh"
 #include "profile.cuh"
+#include "tma.cuh"
 
 #include <cudaTypedefs.h>
 
@@ -379,7 +380,25 @@ PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 std::once_flag g_encode_once;
 }  // namespace
 
-static int encode_2d(CUtensorMap* map, const float* base, int inner, int outer, int pitch,
+int tma_encode_ready() {
+  std::call_once(g_encode_once, [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
+                                         &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+    else
+      cudaGetLastError();
+  });
+  if (!g_encode) {
+    set_error("cuTensorMapEncodeTiled is not available");
+    return LOGDET_ECUDA;
+  }
+  return LOGDET_OK;
+}
+
+int tma_encode_2d(CUtensorMap* map, const float* base, int inner, int outer, int pitch,
                      int box_inner, int box_outer) {
   const cuuint64_t dims[2] = {(cuuint64_t)inner, (cuuint64_t)outer};
   const cuuint64_t strides[1] = {(cuuint64_t)pitch * sizeof(float)};
@@ -398,7 +417,7 @@ static int encode_2d(CUtensorMap* map, const float* base, int inner, int outer, 
 
 // 4D map of an L x ny x nz grid of rows of `inner` floats (pitch floats
 // apart), box of box_inner x bx x by x 1.
-static int encode_grid(CUtensorMap* map, const float* base, const DiaInfo& d, int inner,
+int tma_encode_grid(CUtensorMap* map, const float* base, const DiaInfo& d, int inner,
                        int pitch, int box_inner, int bx, int by) {
   const cuuint64_t dims[4] = {(cuuint64_t)inner, (cuuint64_t)d.L, (cuuint64_t)d.ny,
                               (cuuint64_t)d.nz};
@@ -418,20 +437,7 @@ static int encode_grid(CUtensorMap* map, const float* base, const DiaInfo& d, in
 }
 
 int dia_encode(SpmmJob<float>& J, const float* x, int n, int ld, int width) {
-  std::call_once(g_encode_once, [] {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
-                                         &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-    else
-      cudaGetLastError();
-  });
-  if (!g_encode) {
-    set_error("cuTensorMapEncodeTiled is not available");
-    return LOGDET_ECUDA;
-  }
+  LD_TRY(tma_encode_ready());
   const DiaInfo& d = J.dinfo;
   const int T = J.dia_T;
   const int dp = dia_pad(d.ndiag);
@@ -450,78 +456,12 @@ int dia_encode(SpmmJob<float>& J, const float* x, int n, int ld, int width) {
     return LOGDET_EINVAL;
   }
   if (grid3) {
-    LD_TRY(encode_grid(&J.tmap, x, d, ld, ld, width, bx, by));
-    return encode_grid(&J.vmap, J.dia, d, dp, dp, dp, J.dia_tx, J.dia_ty);
+    LD_TRY(tma_encode_grid(&J.tmap, x, d, ld, ld, width, bx, by));
+    return tma_encode_grid(&J.vmap, J.dia, d, dp, dp, dp, J.dia_tx, J.dia_ty);
   }
-  LD_TRY(encode_2d(&J.tmap, x, ld, n, ld, width, box_rows));
-  return encode_2d(&J.vmap, J.dia, dp, n, dp, dp, T);
+  LD_TRY(tma_encode_2d(&J.tmap, x, ld, n, ld, width, box_rows));
+  return tma_encode_2d(&J.vmap, J.dia, dp, n, dp, dp, T);
 }
-
-// ---------------------------------------------------------------------------
-// TMA and mbarrier helpers (inline PTX)
-// ---------------------------------------------------------------------------
-// A wait gives up after wait_ns of the global timer (2 s in normal use), or
-// after kDiaWaitPolls polls whatever the timer says.
-constexpr int kDiaWaitPolls = 1 << 24;
-constexpr unsigned long long kDiaWaitNs = 2000000000ull;
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t phase) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(bar), "r"(phase)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-// Bounded wait for the barrier's phase to complete.
-__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t phase,
-                                                  unsigned long long wait_ns) {
-  if (mbar_try_wait(bar, phase)) return true;
-  const unsigned long long t0 = global_ns();
-  for (int i = 0; i < kDiaWaitPolls; i += 32) {
-    for (int k = 0; k < 32; ++k)
-      if (mbar_try_wait(bar, phase)) return true;
-    if (global_ns() - t0 > wait_ns) return false;
-  }
-  return false;
-}
-// 4D tiled copy of the box at (column, x, y, z) into shared memory.
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int c, int x,
-                                            int y, int z, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c), "r"(x), "r"(y), "r"(z), "r"(bar)
-      : "memory");
-}
-
-// 2D tiled copy of the box at (x = column, y = row) into shared memory.
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y,
-                                            uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-      : "memory");
-}
-
 
 // ---------------------------------------------------------------------------
 // Units.  Unit u of a job covers segment u % nseg (rows seg0 .. seg0 + segT

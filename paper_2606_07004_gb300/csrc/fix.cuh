@@ -1,0 +1,46 @@
+// Fixed-point form of the FP64 SpMM pass for grid stencil matrices (see
+// fix.cu).
+#pragma once
+
+#include "handle.cuh"
+#include "krylov.cuh"
+
+namespace ld {
+
+// Blocks smaller than this keep the CSR pass: their steps are bound by the
+// latency of dependent launches, not by the FP64 pipe (a 64 x 64 grid's pass
+// takes 4 us of which the pipe is busy 0.8).
+constexpr size_t kFixMinBlock = (size_t)16 << 20;
+
+// Geometry of a slice of `width` columns of an FP64 block; false when the matrix has no
+// grid structure or the slice does not fit.
+struct FixGeom {
+  int T, kc, nseg, nlines, units, tx, ty, txs;
+};
+bool fix_geom(const logdet_ctx* h, int width, int ld, FixGeom* g);
+
+// Whether every row's absolute sum is within 8 of the largest.  The results'
+// unit follows the largest row, so a much smaller row would lose that many
+// bits: with one row 4e5 times heavier than the others the forms moved by
+// 1e-9.
+inline bool fix_balanced(const logdet_ctx* h, double shift) {
+  return std::max(h->g_hi, -h->g_lo) + shift <= 8.0 * (h->row_min + shift);
+}
+
+// Values of (Q + shift I) / c per row and diagonal, [n][ndiag], as fixed-point
+// numbers A 2^(ka - 60), A = hi 2^30 + lo with |lo| <= 2^29; ka from fix_scale.
+int fix_scale(const logdet_ctx* h, double c, double shift);
+int fix_values(const logdet_ctx* h, double c, double shift, int ka, int2* out, cudaStream_t st);
+
+// A job's fixed-point fields (fix, ka, hn, bad) and tensor map from its x,
+// ld, col_off and width; sig / sig_stride / xexp are the caller's.
+int fix_job(SpmmJob<double>& J, const logdet_ctx* h, const FixGeom& g, const int2* fix, int ka,
+            int* bad);
+// One product y = A x over a block whose entries are below 2^xexp in
+// magnitude (no dots).
+int fix_spmm_block(const logdet_ctx* h, const int2* fix, int ka, const double* x, double* y, int ld,
+                   int xexp, cudaStream_t st);
+// Batched launch (all jobs with fix != nullptr and one grid dimension).
+int launch_spmm_fix(const SpmmBatch<double>& b, cudaStream_t s);
+
+}  // namespace ld

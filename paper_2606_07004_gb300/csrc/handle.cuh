@@ -18,6 +18,7 @@ struct logdet_ctx {
   int vals_dtype = LOGDET_VALS_F64;
   bool owns = false;
   double g_lo = 0.0, g_hi = 0.0;  // Gershgorin interval (unclamped)
+  double row_min = 0.0;           // least absolute row sum (CSR)
   cudaStream_t stream = nullptr;
   // Irregular sparsity (some row longer than kSplitRowNnz): a host copy of
   // rowptr and, per tile depth, the SpMM work-item list built from it.

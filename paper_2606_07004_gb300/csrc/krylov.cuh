@@ -74,6 +74,14 @@ struct SpmmJob {
   int* err;
   int dia_T, dia_kc, dia_nseg, dia_nlines;
   int dia_tx, dia_ty, dia_txs;     // plane sweep: tile of tx (= 1 << txs) x ty points, T = tx ty
+  // Fixed-point sweep (FP64 blocks of such a matrix, see fix.cu): the entries
+  // [n][ndiag]; a column of x is scaled by sigma (sig[p * sig_stride], with
+  // hn = floor(log2(n) / 2)) or, without sig, by 2^xexp; bad: set when an
+  // entry of x does not fit.
+  const int2* fix;
+  const double* sig;
+  int* bad;
+  int sig_stride, xexp, hn, ka;
   DiaInfo dinfo;
   CUtensorMap tmap;
   CUtensorMap vmap;

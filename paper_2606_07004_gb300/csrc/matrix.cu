@@ -122,9 +122,9 @@ template <typename V>
 __global__ void k_gershgorin(const int* __restrict__ rowptr, const int* __restrict__ colind,
                              const V* __restrict__ vals, int n, long long nnz,
                              double* __restrict__ lo_out, double* __restrict__ hi_out,
-                             int* __restrict__ flags) {
-  __shared__ double slo[256], shi[256];
-  double lo = INFINITY, hi = -INFINITY;
+                             double* __restrict__ min_out, int* __restrict__ flags) {
+  __shared__ double slo[256], shi[256], smn[256];
+  double lo = INFINITY, hi = -INFINITY, mn = INFINITY;  // mn: the least absolute row sum
   int fl = 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int p0 = rowptr[i], p1 = rowptr[i + 1];
@@ -144,44 +144,50 @@ __global__ void k_gershgorin(const int* __restrict__ rowptr, const int* __restri
     if (!has_d) fl |= 2;
     lo = fmin(lo, d - R);
     hi = fmax(hi, d + R);
+    mn = fmin(mn, fabs(d) + R);
   }
   slo[threadIdx.x] = lo;
   shi[threadIdx.x] = hi;
+  smn[threadIdx.x] = mn;
   __syncthreads();
   for (int w = blockDim.x / 2; w > 0; w >>= 1) {
     if (threadIdx.x < w) {
       slo[threadIdx.x] = fmin(slo[threadIdx.x], slo[threadIdx.x + w]);
       shi[threadIdx.x] = fmax(shi[threadIdx.x], shi[threadIdx.x + w]);
+      smn[threadIdx.x] = fmin(smn[threadIdx.x], smn[threadIdx.x + w]);
     }
     __syncthreads();
   }
   if (threadIdx.x == 0) {
     lo_out[blockIdx.x] = slo[0];
     hi_out[blockIdx.x] = shi[0];
+    min_out[blockIdx.x] = smn[0];
   }
   if (fl) atomicOr(flags, fl);
 }
 
 static int compute_gershgorin(logdet_ctx* h, bool check_structure) {
   const int blocks = std::max(1, std::min(div_up(h->n, 256), 4 * sm_count()));
-  DevBuf<double> lo(h->stream), hi(h->stream);
+  DevBuf<double> lo(h->stream), hi(h->stream), mn(h->stream);
   DevBuf<int> fl(h->stream);
   LD_TRY(lo.alloc(blocks));
   LD_TRY(hi.alloc(blocks));
+  LD_TRY(mn.alloc(blocks));
   LD_TRY(fl.alloc(1));
   LD_CUDA(cudaMemsetAsync(fl.p, 0, sizeof(int), h->stream));
   ProfScope prof(KC_OTHER, h->stream);
   if (h->vals_dtype == LOGDET_VALS_F64)
     k_gershgorin<double><<<blocks, 256, 0, h->stream>>>(h->rowptr, h->colind, (const double*)h->vals,
-                                                       h->n, h->nnz, lo.p, hi.p, fl.p);
+                                                       h->n, h->nnz, lo.p, hi.p, mn.p, fl.p);
   else
     k_gershgorin<float><<<blocks, 256, 0, h->stream>>>(h->rowptr, h->colind, (const float*)h->vals,
-                                                      h->n, h->nnz, lo.p, hi.p, fl.p);
+                                                      h->n, h->nnz, lo.p, hi.p, mn.p, fl.p);
   LD_CHECK_LAUNCH();
-  std::vector<double> hl(blocks), hh(blocks);
+  std::vector<double> hl(blocks), hh(blocks), hm(blocks);
   int hf = 0;
   LD_CUDA(cudaMemcpyAsync(hl.data(), lo.p, sizeof(double) * blocks, cudaMemcpyDeviceToHost, h->stream));
   LD_CUDA(cudaMemcpyAsync(hh.data(), hi.p, sizeof(double) * blocks, cudaMemcpyDeviceToHost, h->stream));
+  LD_CUDA(cudaMemcpyAsync(hm.data(), mn.p, sizeof(double) * blocks, cudaMemcpyDeviceToHost, h->stream));
   LD_CUDA(cudaMemcpyAsync(&hf, fl.p, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   LD_CUDA(cudaStreamSynchronize(h->stream));
   if (check_structure && hf) {
@@ -193,6 +199,7 @@ static int compute_gershgorin(logdet_ctx* h, bool check_structure) {
   for (int b = 0; b < blocks; ++b) { glo = std::min(glo, hl[b]); ghi = std::max(ghi, hh[b]); }
   h->g_lo = glo;
   h->g_hi = ghi;
+  h->row_min = *std::min_element(hm.begin(), hm.end());
   if (!(ghi > 0.0)) {
     set_error("Gershgorin upper bound %g <= 0: matrix is not SPD", ghi);
     return LOGDET_ENOTSPD;

@@ -186,6 +186,13 @@ int KRun<T>::init(const int* rp, const int* ci, const typename ValOf<T>::type* v
       nslots = sg.units;
     }
   }
+  if constexpr (std::is_same<T, double>::value) {
+    // Fixed-point sweep (the solve has checked that every width fits).
+    if (fixvals && fix_geom(hctx, width, ld, &fg)) {
+      sweep = true;
+      nslots = fg.units;
+    }
+  }
   blk = (size_t)n * ld;
   const int win = method == 0 ? 2 : k;
   if (method == 1 && win > kMaxWin - 1) {
@@ -200,8 +207,8 @@ int KRun<T>::init(const int* rp, const int* ci, const typename ValOf<T>::type* v
   // covers (beyond it the norm runs right after its pass, from part).
   if (method != 0 && (size_t)2 * ld * ntiles * sizeof(Part) <= kNormPartMax)
     LD_TRY(npart.alloc((size_t)2 * ld * ntiles));
-  if (diavals) {
-    LD_TRY(dia_err.alloc(1));
+  if (diavals || fixvals) {
+    LD_TRY(dia_err.alloc(2));
     LD_TRY(dia_err.zero());
   }
   LD_TRY(y.alloc(blk));
@@ -277,6 +284,13 @@ int KRun<T>::spmm_jobs(int j, std::vector<SpmmJob<T>>& out) const {
         J.dia_txs = sw_txs;
         J.dinfo = hctx->dia;
         LD_TRY(dia_encode(J, ptr(j), n, ld, width));
+      }
+    }
+    if constexpr (std::is_same<T, double>::value) {
+      if (sweep) {
+        J.sig = ks.sig.p + j;
+        J.sig_stride = m + 2;
+        LD_TRY(fix_job(J, hctx, fg, fixvals, fix_ka, dia_err.p));
       }
     }
     out.push_back(J);
@@ -357,7 +371,7 @@ ScalarJob KRun<T>::scalar_job(int j, int ndots, bool spmm_pass) const {
   ScalarJob sj;
   memset(&sj, 0, sizeof sj);
   sj.st = ks.st;
-  sj.part = part.p;
+  sj.part = spmm_pass || j == 0 ? part.p : norm_part();  // (step 0: the start block's norms)
   sj.part_f32 = std::is_same<T, double>::value ? 0 : 1;
   sj.ntiles = spmm_pass ? nslots : ntiles;
   sj.step = j;
@@ -444,10 +458,10 @@ template struct KRun<f32x2>;
 // ---------------------------------------------------------------------------
 template <typename T>
 int launch_spmm_jobs(const std::vector<SpmmJob<T>>& jobs, int threads, cudaStream_t s) {
-  if constexpr (std::is_same<T, float>::value) {
+  if constexpr (std::is_same<T, float>::value || std::is_same<T, double>::value) {
     // Sweep jobs launch apart from CSR jobs, line sweeps apart from plane
     // sweeps (same stream, in order).
-    auto kind = [](const SpmmJob<T>& J) { return J.dia ? J.dinfo.dim : 0; };
+    auto kind = [](const SpmmJob<T>& J) { return J.dia || J.fix ? J.dinfo.dim : 0; };
     bool mixed = false;
     for (const auto& J : jobs) mixed |= kind(J) != kind(jobs[0]);
     if (mixed) {
@@ -474,6 +488,12 @@ int launch_spmm_jobs(const std::vector<SpmmJob<T>>& jobs, int threads, cudaStrea
     if constexpr (std::is_same<T, float>::value) {
       if (B.jobs[0].dia) {
         LD_TRY(launch_spmm_dia(B, threads, s));
+        continue;
+      }
+    }
+    if constexpr (std::is_same<T, double>::value) {
+      if (B.jobs[0].fix) {
+        LD_TRY(launch_spmm_fix(B, s));
         continue;
       }
     }
@@ -632,6 +652,8 @@ struct Solve : ISolve {
   DevBuf<typename Compute<T>::type> gtabs;  // gridded operator: scaled table (or transform tables)
   GridFft gfft;                              //   the transforms' cover, if they are used
   DevBuf<float> diav;                        // FP32 values per diagonal (diagonal fast path)
+  DevBuf<int2> fixv;                         // fixed-point entries in place of vals (FP64 sweep)
+  int fix_ka = 0;
   DevBuf<T> Vst, Xc;
   DevBuf<double> X64, outv, cshift;
   DevBuf<int> keep;
@@ -653,7 +675,7 @@ struct Solve : ISolve {
   int vst_ld = 0;                //   basis blocks (leading dimension vst_ld)
 
   Solve(logdet_ctx* h_, const SolveCfg& c_, cudaStream_t st_)
-      : h(h_), c(c_), st(st_), vals(st_), gtabs(st_), diav(st_), Vst(st_), Xc(st_), X64(st_), outv(st_), cshift(st_),
+      : h(h_), c(c_), st(st_), vals(st_), gtabs(st_), diav(st_), fixv(st_), Vst(st_), Xc(st_), X64(st_), outv(st_), cshift(st_),
         keep(st_) {
     n = h->n;
     s = c.plain ? 0 : c.P / 3;
@@ -732,7 +754,7 @@ struct Solve : ISolve {
             [&b] { b.release(); }, [&b] { return b.alloc(b.count); }};
   }
   std::vector<BufRef> buffers() {
-    std::vector<BufRef> v = {ref(vals), ref(gtabs), ref(diav), ref(Vst), ref(Xc),
+    std::vector<BufRef> v = {ref(vals), ref(gtabs), ref(diav), ref(fixv), ref(Vst), ref(Xc),
                              ref(X64),  ref(outv),  ref(cshift), ref(keep)};
     if (run) {
       KRun<T>& R = *run;
@@ -804,6 +826,7 @@ struct Solve : ISolve {
       fix(R.colshift);
       fix(R.colscale);
       fix(R.diavals);
+      fix(R.fixvals);
       fix(R.gtab);
       KrylovState& S = R.ks.st;
       fix(S.alpha);
@@ -846,7 +869,7 @@ struct Solve : ISolve {
       tc->split = w / std::min(c.block_width, w);
       return LOGDET_OK;
     }
-    if (!c.autotune) return LOGDET_OK;
+    if (!c.autotune || fixv.p) return LOGDET_OK;  // (the fixed-point sweep has one layout)
     const int nd = c.method == 0 ? 1 : kk, nb = c.method == 0 ? 2 : kk;
     return autotune_krylov<T>(h, vals.p, w, nd, nb, track_e ? 1 : 0,
                               st, tc);
@@ -867,6 +890,20 @@ struct Solve : ISolve {
   }
 
   double cscale() const { return c.method == 0 ? alpha : gamma; }
+  // FP64 blocks of a grid stencil, above kFixMinBlock: pass 1 in fixed point
+  // (group members share one run whose columns have factors of their own, and
+  // keep the CSR pass).
+  bool use_fix() const {
+    if (!std::is_same<T, double>::value || grouped || h->kind != 0) return false;
+    const int narrow = s ? std::min(ld, lds) : ld;
+    if ((size_t)n * narrow * sizeof(double) <= kFixMinBlock || !fix_balanced(h, c.shift)) return false;
+    FixGeom g;
+    for (int w : {ld, s ? lds : ld}) {
+      if (!fix_geom(h, w, w, &g)) return false;
+      if (c.block_width > 0 && !fix_geom(h, std::min(c.block_width, w), w, &g)) return false;
+    }
+    return true;
+  }
   // Group member: free the start block once the group has copied it.
   void release_start() {
     if (pend_x0 == Vst.p) Vst.release();
@@ -949,6 +986,10 @@ struct Solve : ISolve {
           LD_TRY(grid_table<typename Compute<T>::type>(h, cscale, gtabs.p, st));
         }
       }
+    } else if (use_fix()) {
+      fix_ka = fix_scale(h, cscale, c.shift);
+      LD_TRY(fixv.alloc((size_t)h->dia.ndiag * n));
+      LD_TRY(fix_values(h, cscale, c.shift, fix_ka, fixv.p, st));
     } else {
       LD_TRY(vals.alloc(h->nnz));
       LD_TRY(scaled_values<typename ValOf<T>::type>(h, cscale, vals.p, st));
@@ -975,6 +1016,8 @@ struct Solve : ISolve {
       run->gtab = gtabs.p;
       run->gfft = gfft;
       run->diavals = diav.p;
+      run->fixvals = fixv.p;
+      run->fix_ka = fix_ka;
       TuneCfg tc;
       LD_TRY(layout(ld, c.method == 1, &tc));
       if (c.method == 0) {
@@ -998,6 +1041,7 @@ struct Solve : ISolve {
         if (h->kind == 1 && gfft.pairs)
           LD_TRY(grid_fft_apply<T>(h, gfft, gtabs.p, S.p, Yt.p, lds, cshift.p, nullptr, 0, st));
         else if (h->kind == 1) LD_TRY(grid_apply<T>(h, gtabs.p, S.p, Yt.p, lds, cshift.p, st));
+        else if (fixv.p) LD_TRY(sketch_fix(S.p, Yt.p));
         else LD_TRY(spmm_block<T>(h->rowptr, h->colind, vals.p, n, S.p, Yt.p, lds, st, cshift.p, h));
       }
       S.release();
@@ -1025,6 +1069,8 @@ struct Solve : ISolve {
       run->gtab = gtabs.p;
       run->gfft = gfft;
       run->diavals = diav.p;
+      run->fixvals = fixv.p;
+      run->fix_ka = fix_ka;
       TuneCfg tc;
       LD_TRY(layout(ld, false, &tc));
       LD_TRY(start_run(b, ld, 2, 0, false, X0, nullptr, tc));
@@ -1038,12 +1084,23 @@ struct Solve : ISolve {
       run->gtab = gtabs.p;
       run->gfft = gfft;
       run->diavals = diav.p;
+      run->fixvals = fixv.p;
+      run->fix_ka = fix_ka;
       TuneCfg tc;
       LD_TRY(layout(lds, false, &tc));
       LD_TRY(start_run(s, lds, kk, 1, false, Vst.p, Vst.p, tc));
     }
     ph = PH_K1;
     return LOGDET_OK;
+  }
+
+  // The sketch product in fixed point: probe entries are +-1, or Gaussian
+  // (below 9 from 53-bit uniforms).
+  int sketch_fix(const T* S, T* Y) {
+    if constexpr (std::is_same<T, double>::value)
+      return fix_spmm_block(h, fixv.p, fix_ka, S, Y, lds, 4, st);
+    else
+      return LOGDET_EINVAL;
   }
 
   int mid() {
@@ -1085,6 +1142,8 @@ struct Solve : ISolve {
     run->gtab = gtabs.p;
     run->gfft = gfft;
     run->diavals = diav.p;
+    run->fixvals = fixv.p;
+    run->fix_ka = fix_ka;
     TuneCfg tc;
     LD_TRY(layout(ld, true, &tc));
     LD_TRY(start_run(b, ld, kk, 1, true, X0, nullptr, tc));
@@ -1123,6 +1182,7 @@ struct Solve : ISolve {
     vals.release();
     gtabs.release();
     diav.release();
+    fixv.release();
     cshift.release();
     X64.release();
     Xc.release();

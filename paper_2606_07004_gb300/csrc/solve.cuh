@@ -16,6 +16,7 @@
 #pragma once
 
 #include "dense.cuh"
+#include "fix.cuh"
 #include "grid.cuh"
 #include "handle.cuh"
 #include "krylov.cuh"
@@ -107,7 +108,10 @@ struct KRun {
   DevBuf<T> y, ring;
   KState ks;
   const float* diavals = nullptr;  // FP32 values per row and diagonal: the line-sweep path
-  DevBuf<int> dia_err;             // set if a staged copy's wait gave up
+  const int2* fixvals = nullptr;   // fixed-point entries: the FP64 sweep (fix.cu), their scale
+  int fix_ka = 0;
+  FixGeom fg{};
+  DevBuf<int> dia_err;             // [0] set if a staged copy's wait gave up; [1] fixed-point range
   bool sweep = false;              // pass 1 runs the line sweep
   int sw_T = 0, sw_kc = 0, sw_nseg = 0, sw_nlines = 0, sw_tx = 0, sw_ty = 0, sw_txs = 0;
   int done_steps = 0;  // steps whose pass 1 has been issued
@@ -132,7 +136,8 @@ struct KRun {
   Part* norm_part() const {
     return method == 0 ? part.p + (size_t)ld * std::max(ntiles, nslots) : npart.p ? npart.p : part.p;
   }
-  bool late_norm() const { return method == 0 || npart.p; }
+  // (the fixed-point sweep scales its input by sigma_j, so it needs the norm)
+  bool late_norm() const { return (method == 0 || npart.p) && !(sweep && fixvals); }
   // Step j's jobs, one per column slice.
   int spmm_jobs(int j, std::vector<SpmmJob<T>>& out) const;
   // Gridded operator: step j's pass 1 (y = Q~ u_j and the window dots),
