@@ -1,11 +1,13 @@
 // Dense and small-matrix kernels (see dense.cuh).  Arithmetic is FP64, except
 // the FP32 instances of the Hutch++ split kernels (mixed-precision OSLQ).
 #include "dense.cuh"
+#include "densefix.cuh"
 #include "krylov.cuh"
 #include "profile.cuh"
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 namespace ld {
@@ -17,7 +19,14 @@ namespace ld {
 // Householder QR with that sign convention.
 // ===========================================================================
 constexpr int kGramThreads = 256;
-constexpr int kGramRows = 256;   // rows per tile (one partial per tile)
+// Rows per tile (one partial per tile): 256, or fewer where those leave SMs
+// without a tile: a tile is a chain of dependent FP64 multiply-adds (4,096
+// rows, 10 columns: 33.7 us a Gram with 16 tiles).
+inline int gram_rows(int n) {
+  int rows = 256;
+  while (rows > 32 && n < rows * sm_count()) rows /= 2;
+  return rows;
+}
 constexpr int kGramChunk = 32;   // rows staged in shared memory at a time
 
 __device__ __forceinline__ void unrank_upper(int q, int s, int& i, int& j) {
@@ -42,8 +51,10 @@ template <> struct GramAcc<float> { using type = AccF; };
 // written).
 template <int NP, typename TY>
 __global__ void __launch_bounds__(kGramThreads) k_gram(const TY* __restrict__ Y, int ldy,
-                                                       int n, int s, int ntiles,
-                                                       double* __restrict__ part) {
+                                                       int n, int s, int ntiles, int tile_rows,
+                                                       double* __restrict__ part,
+                                                       const int* __restrict__ run) {
+  if (run && !*run) return;
   __shared__ double sy_raw[kGramChunk * kMaxSketch];
   TY* sy = reinterpret_cast<TY*>(sy_raw);
   // Rows staged at a time: the buffer's capacity for s columns (32 for the
@@ -61,8 +72,8 @@ __global__ void __launch_bounds__(kGramThreads) k_gram(const TY* __restrict__ Y,
     typename GramAcc<TY>::type acc[NP];
 #pragma unroll
     for (int q = 0; q < NP; ++q) acc[q].zero();
-    const int row0 = tile * kGramRows;
-    const int row1 = min(row0 + kGramRows, n);
+    const int row0 = tile * tile_rows;
+    const int row1 = min(row0 + tile_rows, n);
     for (int c0 = row0; c0 < row1; c0 += chunk) {
       const int rows = min(chunk, row1 - c0);
       __syncthreads();
@@ -87,9 +98,12 @@ __global__ void __launch_bounds__(kGramThreads) k_gram(const TY* __restrict__ Y,
 
 // Sum the tile partials of each entry in a fixed order: out[e] for e < count.
 // With sym_s > 0 the entries are upper-triangle pairs of an sym_s x sym_s
-// matrix and both (i,j) and (j,i) of out are written.
+// matrix and both (i,j) and (j,i) of out are written.  With bad (a block that
+// may have taken the fixed-point sums) there are nfix partials unless it is set.
 __global__ void __launch_bounds__(128) k_reduce_rows(const double* __restrict__ part, int ntiles,
-                                                     int sym_s, double* __restrict__ out) {
+                                                     int sym_s, double* __restrict__ out,
+                                                     const int* __restrict__ bad, int nfix) {
+  if (bad && !*bad) ntiles = nfix;
   __shared__ double sh[128];
   const int e = blockIdx.x;
   const double* src = part + (size_t)e * ntiles;
@@ -115,55 +129,45 @@ __global__ void __launch_bounds__(128) k_reduce_rows(const double* __restrict__ 
 
 // Cholesky C = R^T R of the s x s Gram matrix, dropping a column whose pivot
 // R_jj^2 is <= thr_rel * max_i C_ii (its R row and Rinv column become zero),
-// then Rinv = R^{-1} restricted to the kept columns.  One CTA.
+// and Rinv = R^{-1} restricted to the kept columns.  One CTA: step j scales
+// row j by the reciprocal root of its pivot and subtracts its multiples from
+// the rows below, in the upper triangle (C becoming R) and, as a Gauss-Jordan
+// elimination of the identity, in the lower one (column c <= j of row i holds
+// the rows of R^{-T} so far), so that a step is two short parallel passes;
+// one thread's dot products for each pivot, and one a column for the inverse,
+// took 55 us at s = 20 and 160 us at s = 40.
 __global__ void __launch_bounds__(256) k_chol_inv(const double* __restrict__ C, int s,
                                                   double thr_rel, double* __restrict__ Rinv,
                                                   int* __restrict__ keep_out) {
-  __shared__ double R[kMaxSketch * kMaxSketch];
-  __shared__ int keep[kMaxSketch];
-  __shared__ double thr;
-  double* Ri = Rinv;  // written column by column by the thread that owns it
-  for (int e = threadIdx.x; e < s * s; e += blockDim.x) { R[e] = C[e]; Ri[e] = 0.0; }
+  __shared__ double M[kMaxSketch * kMaxSketch];
+  for (int e = threadIdx.x; e < s * s; e += blockDim.x) M[e] = C[e];
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double mx = 0.0;
-    for (int i = 0; i < s; ++i) mx = fmax(mx, R[i * s + i]);
-    thr = thr_rel * mx;
-  }
-  __syncthreads();
+  double mx = 0.0;
+  for (int i = 0; i < s; ++i) mx = fmax(mx, M[i * s + i]);
+  const double thr = thr_rel * mx;
   for (int j = 0; j < s; ++j) {
-    if (threadIdx.x == 0) {
-      double piv = R[j * s + j];
-      for (int k = 0; k < j; ++k) piv -= R[k * s + j] * R[k * s + j];
-      keep[j] = piv > thr;
-      R[j * s + j] = keep[j] ? sqrt(piv) : 0.0;
+    __syncthreads();
+    const double piv = M[j * s + j];
+    const bool kept = piv > thr;
+    __syncthreads();
+    if (threadIdx.x < s) {
+      const int c = threadIdx.x;
+      const double inv = kept ? rsqrt(piv) : 0.0;
+      M[j * s + c] = !kept ? 0.0 : c == j ? inv : M[j * s + c] * inv;
+      if (c == j) keep_out[j] = kept;
     }
     __syncthreads();
-    for (int l = j + 1 + threadIdx.x; l < s; l += blockDim.x) {
-      if (keep[j]) {
-        double v = R[j * s + l];
-        for (int k = 0; k < j; ++k) v -= R[k * s + j] * R[k * s + l];
-        R[j * s + l] = v / R[j * s + j];
-      } else {
-        R[j * s + l] = 0.0;
-      }
+    for (int e = threadIdx.x; e < (s - 1 - j) * s; e += blockDim.x) {
+      const int q = e / s, c = e - q * s, i = j + 1 + q;
+      if (c > j && c < i) continue;
+      M[i * s + c] = fma(-M[j * s + i], M[j * s + c], c == j ? 0.0 : M[i * s + c]);
     }
-    __syncthreads();
   }
-  // Upper-triangular inverse, one column per thread: R Rinv = I.  The zero
-  // fill above is made visible to every thread before columns are written.
-  __threadfence_block();
   __syncthreads();
-  for (int l = threadIdx.x; l < s; l += blockDim.x) {
-    if (!keep[l]) continue;
-    for (int i = l; i >= 0; --i) {
-      if (!keep[i]) { Ri[i * s + l] = 0.0; continue; }
-      double v = (i == l) ? 1.0 : 0.0;
-      for (int k = i + 1; k <= l; ++k) v -= R[i * s + k] * Ri[k * s + l];
-      Ri[i * s + l] = v / R[i * s + i];
-    }
+  for (int e = threadIdx.x; e < s * s; e += blockDim.x) {
+    const int i = e / s, l = e - i * s;
+    Rinv[e] = i <= l ? M[l * s + i] : 0.0;
   }
-  for (int i = threadIdx.x; i < s; i += blockDim.x) keep_out[i] = keep[i];
 }
 
 // A[row, l] = sum_{i <= l} Y[row, i] Rinv[i, l]; A may alias Y.  A chunk of
@@ -179,7 +183,8 @@ constexpr int kApplyCols = 4;
 template <typename TY>
 __global__ void __launch_bounds__(512) k_apply_rinv(const TY* Y, int ldy, int n, int s,
                                                     const double* __restrict__ Rinv, TY* A,
-                                                    int lda) {
+                                                    int lda, const int* __restrict__ run) {
+  if (run && !*run) return;
   extern __shared__ double smem_ar[];
   const int S1 = s | 1;
   TY* sr = reinterpret_cast<TY*>(smem_ar);
@@ -214,9 +219,10 @@ __global__ void __launch_bounds__(512) k_apply_rinv(const TY* Y, int ldy, int n,
 }
 
 size_t orth_workspace_doubles(int n, int s) {
-  int ntiles = div_up(n, kGramRows);
+  int ntiles = div_up(n, gram_rows(n));
   size_t npairs = (size_t)s * (s + 1) / 2;
-  return npairs * ntiles + 2 * (size_t)s * s + 64;
+  return npairs * ntiles + 2 * (size_t)s * s + 64 +
+         (densefix_ok(n, s) ? densefix_workspace_doubles(s) : 0);
 }
 
 // Persistent grids: 4 CTAs per SM, or for CTAs of fewer than 256 threads
@@ -249,7 +255,7 @@ static int pairs_instance(int per) {
 }
 
 template <typename TY>
-using GramKern = void (*)(const TY*, int, int, int, int, double*);
+using GramKern = void (*)(const TY*, int, int, int, int, int, double*, const int*);
 template <typename TY>
 static GramKern<TY> gram_kernel(int np) {
   switch (np) {
@@ -270,11 +276,13 @@ static int orth_t(int n, int s, const TY* Y, int ldy, TY* A, int lda, double* ws
     set_error("orth: s=%d must be in [1, %d]", s, kMaxSketch);
     return LOGDET_EINVAL;
   }
-  const int ntiles = div_up(n, kGramRows);
+  const int tile_rows = gram_rows(n), ntiles = div_up(n, tile_rows);
   const int npairs = s * (s + 1) / 2;
   double* part = ws;
   double* C = part + (size_t)npairs * ntiles;
   double* Rinv = C + (size_t)s * s;
+  const bool fix = densefix_ok(n, s);
+  ColScales cs;
   int* keep = keep_dev;
   int* keep_tmp = nullptr;
   if (!keep) {
@@ -299,16 +307,29 @@ static int orth_t(int n, int s, const TY* Y, int ldy, TY* A, int lda, double* ws
     prof_count();
     prof_count();
     prof_count();
+    if (fix) {
+      LD_TRY(column_scales<TY>(src, ldsrc, n, s, Rinv + (size_t)s * s + 64, &cs, st));
+      LD_TRY(gram_fix<TY>(src, ldsrc, n, s, cs, part, st));
+      for (int q = 0; q < 3; ++q) prof_count();
+    }
     gram<<<grid_for(gram, ntiles, gram_threads), gram_threads, 0, st>>>(src, ldsrc, n, s, ntiles,
-                                                                         part);
+                                                                         tile_rows, part, cs.bad);
     LD_CHECK_LAUNCH();
-    k_reduce_rows<<<npairs, 128, 0, st>>>(part, ntiles, s, C);
+    k_reduce_rows<<<npairs, 128, 0, st>>>(part, ntiles, s, C, cs.bad, densefix_slots(n));
     LD_CHECK_LAUNCH();
     // R14: |R_ii| <= 1e-6 max_j |y_j|  <=>  R_ii^2 <= 1e-12 max_j C_jj.
     k_chol_inv<<<1, 256, 0, st>>>(C, s, 1e-12, Rinv, keep);
     LD_CHECK_LAUNCH();
+    const int* run = nullptr;
+    if constexpr (std::is_same<TY, double>::value) {
+      if (fix) {
+        LD_TRY(apply_fix(src, ldsrc, n, s, Rinv, A, lda, cs, st));
+        prof_count();
+        run = cs.bad;
+      }
+    }
     k_apply_rinv<TY><<<grid_for(k_apply_rinv<TY>, div_up(n, 32), apply_threads, apply_smem),
-                       apply_threads, apply_smem, st>>>(src, ldsrc, n, s, Rinv, A, lda);
+                       apply_threads, apply_smem, st>>>(src, ldsrc, n, s, Rinv, A, lda, run);
     LD_CHECK_LAUNCH();
     src = A;
     ldsrc = lda;
@@ -344,8 +365,10 @@ template <int NP, typename TY>
 __global__ void __launch_bounds__(kGramThreads) k_atg(const TY* __restrict__ A, int lda,
                                                       int n, int s, int r, uint64_t key,
                                                       const uint64_t* __restrict__ keyp,
-                                                      int ntiles, double* __restrict__ part,
-                                                      int gaussian) {
+                                                      int ntiles, int tile_rows,
+                                                      double* __restrict__ part, int gaussian,
+                                                      const int* __restrict__ run) {
+  if (run && !*run) return;
   if (keyp) key = *keyp;
   __shared__ double sa_raw[kGramChunk * kMaxSketch];
   __shared__ double sg_raw[kGramChunk * kMaxSketch];
@@ -364,8 +387,8 @@ __global__ void __launch_bounds__(kGramThreads) k_atg(const TY* __restrict__ A, 
     typename GramAcc<TY>::type acc[NP];
 #pragma unroll
     for (int q = 0; q < NP; ++q) acc[q].zero();
-    const int row0 = tile * kGramRows;
-    const int row1 = min(row0 + kGramRows, n);
+    const int row0 = tile * tile_rows;
+    const int row1 = min(row0 + tile_rows, n);
     for (int c0 = row0; c0 < row1; c0 += chunk) {
       const int rows = min(chunk, row1 - c0);
       __syncthreads();
@@ -405,7 +428,9 @@ template <typename TY>
 __global__ void __launch_bounds__(256) k_project(const TY* A, int lda, int n, int s, int r,
                                                  uint64_t key, const uint64_t* __restrict__ keyp,
                                                  const double* __restrict__ Bm,
-                                                 TY* X, int ldx, int zcol0, int gaussian) {
+                                                 TY* X, int ldx, int zcol0, int gaussian,
+                                                 const int* __restrict__ run) {
+  if (run && !*run) return;
   if (keyp) key = *keyp;
   __shared__ double sb_raw[kMaxSketch * kMaxSketch];
   __shared__ double sa_raw[kGramChunk * kMaxSketch];
@@ -433,19 +458,20 @@ __global__ void __launch_bounds__(256) k_project(const TY* A, int lda, int n, in
 
 int reduce_partials_fp64(const double* part, int nrows, int ntiles, double* out, cudaStream_t st) {
   ProfScope prof(KC_SCALAR, st);
-  k_reduce_rows<<<nrows, 128, 0, st>>>(part, ntiles, 0, out);
+  k_reduce_rows<<<nrows, 128, 0, st>>>(part, ntiles, 0, out, nullptr, 0);
   LD_CHECK_LAUNCH();
   return LOGDET_OK;
 }
 
 size_t project_workspace_doubles(int n, int s, int r) {
-  int ntiles = div_up(n, kGramRows);
-  return (size_t)s * r * ntiles + (size_t)s * r + 64;
+  int ntiles = div_up(n, gram_rows(n));
+  return (size_t)s * r * ntiles + (size_t)s * r + 64 +
+         (densefix_ok(n, s) ? densefix_workspace_doubles(s) : 0);
 }
 
 template <typename TY>
-using AtgKern = void (*)(const TY*, int, int, int, int, uint64_t, const uint64_t*, int, double*,
-                         int);
+using AtgKern = void (*)(const TY*, int, int, int, int, uint64_t, const uint64_t*, int, int, double*,
+                         int, const int*);
 template <typename TY>
 static AtgKern<TY> atg_kernel(int np) {
   switch (np) {
@@ -468,9 +494,11 @@ static int project_residual_t(int n, int s, int r, const TY* A, int lda, uint64_
     set_error("project: s=%d r=%d out of range", s, r);
     return LOGDET_EINVAL;
   }
-  const int ntiles = div_up(n, kGramRows);
+  const int tile_rows = gram_rows(n), ntiles = div_up(n, tile_rows);
   double* part = ws;
   double* Bm = ws + (size_t)s * r * ntiles;
+  const bool fix = densefix_ok(n, s) && !gaussian;  // (its sums take probes of +-1)
+  ColScales cs;
   ProfScope prof(KC_PROJECT, st, 4.0 * n * (double)s * r, sizeof(TY) * n * (2.0 * s + r));
   if (s > 0) {
     prof_count();
@@ -479,14 +507,27 @@ static int project_residual_t(int n, int s, int r, const TY* A, int lda, uint64_
     const int np = s * r, per = pairs_instance(div_up(np, kGramThreads));
     const int atg_threads = std::min(kGramThreads, div_up(div_up(np, per), 32) * 32);
     const AtgKern<TY> atg = atg_kernel<TY>(per);
-    atg<<<grid_for(atg, ntiles, atg_threads), atg_threads, 0, st>>>(A, lda, n, s, r, key, keyp,
-                                                                     ntiles, part, gaussian);
+    if (fix) {
+      LD_TRY(column_scales<TY>(A, lda, n, s, Bm + (size_t)s * r + 64, &cs, st));
+      LD_TRY(atg_fix<TY>(A, lda, n, s, r, key, keyp, cs, part, st));
+      for (int q = 0; q < 3; ++q) prof_count();
+    }
+    atg<<<grid_for(atg, ntiles, atg_threads), atg_threads, 0, st>>>(
+        A, lda, n, s, r, key, keyp, ntiles, tile_rows, part, gaussian, cs.bad);
     LD_CHECK_LAUNCH();
-    k_reduce_rows<<<s * r, 128, 0, st>>>(part, ntiles, 0, Bm);
+    k_reduce_rows<<<s * r, 128, 0, st>>>(part, ntiles, 0, Bm, cs.bad, densefix_slots(n));
     LD_CHECK_LAUNCH();
   }
+  const int* run = nullptr;
+  if constexpr (std::is_same<TY, double>::value) {
+    if (fix) {
+      LD_TRY(project_fix(A, lda, n, s, r, key, keyp, Bm, X + zcol0, ldx, cs, st));
+      prof_count();
+      run = cs.bad;
+    }
+  }
   k_project<TY><<<grid_for(k_project<TY>, div_up(n, project_chunk(s))), 256, 0, st>>>(
-      A, lda, n, s, r, key, keyp, Bm, X, ldx, zcol0, gaussian);
+      A, lda, n, s, r, key, keyp, Bm, X, ldx, zcol0, gaussian, run);
   LD_CHECK_LAUNCH();
   return LOGDET_OK;
 }
