@@ -98,7 +98,18 @@ __device__ __forceinline__ double probe_gauss(uint64_t key, uint32_t col, uint32
 }
 
 __device__ __forceinline__ double probe_value(uint64_t key, uint32_t col, uint32_t row, int gaussian) {
-  return gaussian ? probe_gauss(key, col, row) : (double)probe_sign(key, col, row);
+  // (+-1 from its bits: a conversion to FP64 takes the FP64 pipe 64 clocks)
+  return gaussian ? probe_gauss(key, col, row)
+                  : __hiloint2double(0x3ff00000 | (probe_sign(key, col, row) & (int)0x80000000), 0);
+}
+// The same entry rounded to FP32 where TY is float.
+template <typename TY>
+__device__ __forceinline__ TY probe_entry(uint64_t key, uint32_t col, uint32_t row, int gaussian) {
+  if constexpr (sizeof(TY) == 4) {
+    return gaussian ? (TY)probe_gauss(key, col, row) : (TY)probe_sign(key, col, row);
+  } else {
+    return (TY)probe_value(key, col, row, gaussian);
+  }
 }
 
 // ---------------------------------------------------------------------------

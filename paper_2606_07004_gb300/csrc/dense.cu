@@ -281,7 +281,7 @@ static int orth_t(int n, int s, const TY* Y, int ldy, TY* A, int lda, double* ws
   double* part = ws;
   double* C = part + (size_t)npairs * ntiles;
   double* Rinv = C + (size_t)s * s;
-  const bool fix = densefix_ok(n, s);
+  const bool fix = densefix_ok(n, s, std::is_same<TY, float>::value);
   ColScales cs;
   int* keep = keep_dev;
   int* keep_tmp = nullptr;
@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(kGramThreads) k_atg(const TY* __restrict__ A, 
       }
       for (int e = threadIdx.x; e < rows * r; e += blockDim.x) {
         int rr = e / r, j = e - rr * r;
-        sg[rr * r + j] = (TY)probe_value(key, (uint32_t)j, (uint32_t)(c0 + rr), gaussian);
+        sg[rr * r + j] = probe_entry<TY>(key, (uint32_t)j, (uint32_t)(c0 + rr), gaussian);
       }
       __syncthreads();
       const TY* ra = sa;
@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(256) k_project(const TY* A, int lda, int n, in
       int rr = e / r, j = e - rr * r;
       TY acc = TY(0);
       for (int i = 0; i < s; ++i) acc = fma(sa[rr * s + i], sb[i * r + j], acc);
-      TY g = (TY)probe_value(key, (uint32_t)j, (uint32_t)(c0 + rr), gaussian);
+      TY g = probe_entry<TY>(key, (uint32_t)j, (uint32_t)(c0 + rr), gaussian);
       X[(size_t)(c0 + rr) * ldx + zcol0 + j] = g - acc;
     }
   }
@@ -497,7 +497,7 @@ static int project_residual_t(int n, int s, int r, const TY* A, int lda, uint64_
   const int tile_rows = gram_rows(n), ntiles = div_up(n, tile_rows);
   double* part = ws;
   double* Bm = ws + (size_t)s * r * ntiles;
-  const bool fix = densefix_ok(n, s) && !gaussian;  // (its sums take probes of +-1)
+  const bool fix = densefix_ok(n, s, std::is_same<TY, float>::value) && !gaussian;  // (its sums take probes of +-1)
   ColScales cs;
   ProfScope prof(KC_PROJECT, st, 4.0 * n * (double)s * r, sizeof(TY) * n * (2.0 * s + r));
   if (s > 0) {
@@ -1232,9 +1232,12 @@ __global__ void k_probe_fill(uint64_t key, const uint64_t* __restrict__ keyp, in
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
        e += (size_t)gridDim.x * blockDim.x) {
     int row = (int)(e / ld), c = (int)(e - (size_t)row * ld);
-    double v = 0.0;
-    if (c < ncols) v = probe_value(key, (uint32_t)(col0 + c), (uint32_t)row, gaussian);
-    out[e] = cvt<T>(v);
+    // (FP32: no conversion from FP64, which would bound the pass)
+    using P = typename std::conditional<std::is_same<T, float>::value, float, double>::type;
+    P v = P(0);
+    if (c < ncols) v = probe_entry<P>(key, (uint32_t)(col0 + c), (uint32_t)row, gaussian);
+    if constexpr (std::is_same<T, float>::value) out[e] = v;
+    else out[e] = cvt<T>(v);
   }
 }
 

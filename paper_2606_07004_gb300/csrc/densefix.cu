@@ -30,8 +30,11 @@
 //   1M x 40 FP32             610 -> 465                1174 -> 618
 // The integer multiply-adds' pipe bounds the sums (three of them a product, no
 // FP32 part: 200 us at 1M x 20, the pipe 81 % busy); the applies wait at the
-// chunk barrier as well.  Below 2e7 = n s^2 the FP64 sums take less than the
-// four launches more.
+// chunk barrier as well.  The rule (densefix_ok), whole orthogonalisations:
+// FP64 125,000 x 20 (n s^2 = 5e7) 408 -> 224 us, 1M x 10 740 -> 413; FP32
+// 500,000 x 20 (2e8) 430 -> 362 us, but a server's burst of blocks of 1e8 and
+// less, whose launches count (three more a sum), took 28.9 ms with the
+// fixed-point sums and 28.7 without.
 #include "densefix.cuh"
 #include "dense.cuh"
 #include "krylov.cuh"
@@ -551,7 +554,9 @@ int apply_launch(const double* Y, int ldy, int n, int s, int r, const double* Rm
 }
 }  // namespace
 
-bool densefix_ok(int n, int s) { return s > 0 && (double)n * s * s >= 2e7; }
+bool densefix_ok(int n, int s, bool fp32) {
+  return s > 0 && (double)n * s * s >= (fp32 ? 2e8 : 2e7);
+}
 
 size_t densefix_workspace_doubles(int s) { return (size_t)s * 4 * sm_count() + kMaxSketch + 2; }
 

@@ -5,8 +5,9 @@
 
 namespace ld {
 
-// Whether a block of n rows and s columns takes the fixed-point products.
-bool densefix_ok(int n, int s);
+// Whether a block of n rows and s columns takes the fixed-point products (FP32
+// blocks from a larger size).
+bool densefix_ok(int n, int s, bool fp32 = false);
 // Workspace (doubles) of column_scales for s columns.
 size_t densefix_workspace_doubles(int s);
 // Partial slots of gram_fix and atg_fix: at most one per 256 rows.

@@ -262,27 +262,19 @@ int dia_build(logdet_ctx* h, const int* rowptr, const int* colind) {
   return LOGDET_OK;
 }
 
-template <typename V>
 __global__ void k_dia_values(const int* __restrict__ rowptr, const int* __restrict__ slot,
-                             const V* __restrict__ vals, int n, int dp, double c,
-                             float* __restrict__ out) {
+                             const float* __restrict__ vals, int n, int dp, float* __restrict__ out) {
   for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < n; row += gridDim.x * blockDim.x)
-    for (int q = rowptr[row]; q < rowptr[row + 1]; ++q)
-      out[(size_t)row * dp + slot[q]] = (float)((double)vals[q] / c);
+    for (int q = rowptr[row]; q < rowptr[row + 1]; ++q) out[(size_t)row * dp + slot[q]] = vals[q];
 }
 
-int dia_values_f32(const logdet_ctx* h, double c, float* out, cudaStream_t st) {
+int dia_values_f32(const logdet_ctx* h, const float* vals, float* out, cudaStream_t st) {
   const int n = h->n;
   const int dp = dia_pad(h->dia.ndiag);
   LD_CUDA(cudaMemsetAsync(out, 0, sizeof(float) * (size_t)dp * n, st));
   ProfScope prof(KC_OTHER, st);
   const int blocks = std::max(1, std::min(div_up(n, 256), 8 * sm_count()));
-  if (h->vals_dtype == LOGDET_VALS_F64)
-    k_dia_values<double><<<blocks, 256, 0, st>>>(h->rowptr, h->dia_slot, (const double*)h->vals,
-                                                 n, dp, c, out);
-  else
-    k_dia_values<float><<<blocks, 256, 0, st>>>(h->rowptr, h->dia_slot, (const float*)h->vals, n,
-                                                dp, c, out);
+  k_dia_values<<<blocks, 256, 0, st>>>(h->rowptr, h->dia_slot, vals, n, dp, out);
   LD_CHECK_LAUNCH();
   return LOGDET_OK;
 }

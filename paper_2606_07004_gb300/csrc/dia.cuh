@@ -29,9 +29,9 @@ bool dia_detect(int n, const int* rowptr, const int* colind, DiaInfo* out);
 // structure if there is one, else a 3D grid stencil.
 int dia_build(logdet_ctx* h, const int* rowptr, const int* colind);
 
-// Values of Q / c per row and diagonal, [n][dia_pad(ndiag)] (0 where a row
-// has no entry on a diagonal); the division in FP64 as for the CSR values.
-int dia_values_f32(const logdet_ctx* h, double c, float* out, cudaStream_t st);
+// The scaled CSR values per row and diagonal, [n][dia_pad(ndiag)] (0 where a
+// row has no entry on a diagonal).
+int dia_values_f32(const logdet_ctx* h, const float* vals, float* out, cudaStream_t st);
 
 // Sweep geometry of a block slice of `width` FP32 columns processed by CTAs
 // of `threads`: points per segment or tile T (dim 2: a multiple of the row

@@ -993,9 +993,11 @@ struct Solve : ISolve {
     } else {
       LD_TRY(vals.alloc(h->nnz));
       LD_TRY(scaled_values<typename ValOf<T>::type>(h, cscale, vals.p, st));
-      if (std::is_same<T, float>::value && h->dia.ndiag > 0 && h->dia_slot) {
-        LD_TRY(diav.alloc((size_t)dia_pad(h->dia.ndiag) * n));
-        LD_TRY(dia_values_f32(h, cscale, diav.p, st));
+      if constexpr (std::is_same<T, float>::value) {
+        if (h->dia.ndiag > 0 && h->dia_slot) {
+          LD_TRY(diav.alloc((size_t)dia_pad(h->dia.ndiag) * n));
+          LD_TRY(dia_values_f32(h, vals.p, diav.p, st));
+        }
       }
     }
     if (c.shift != 0.0) {

@@ -162,13 +162,12 @@ int autotune_krylov(logdet_ctx* h, const typename ValOf<T>::type* vals, int ld, 
     if (sw_ok && dia_sweep_geom(h, ld / c.split, g.threads, &sg))
       max_slots = std::max(max_slots, sg.units);
   }
-  // Line sweep: FP32 values per row and diagonal (unscaled: only the time
-  // counts) and the wait-failure flag.
+  // Line sweep: FP32 values per row and diagonal and the wait-failure flag.
   DevBuf<float> dvals(st);
   DevBuf<int> derr(st);
   if (sw_ok) {
     LD_TRY(dvals.alloc((size_t)dia_pad(h->dia.ndiag) * n));
-    LD_TRY(dia_values_f32(h, 1.0, dvals.p, st));
+    if constexpr (std::is_same<T, float>::value) LD_TRY(dia_values_f32(h, vals, dvals.p, st));
     LD_TRY(derr.alloc(1));
     LD_TRY(derr.zero());
   }

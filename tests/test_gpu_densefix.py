@@ -1,4 +1,5 @@
-"""The fixed-point products of the Hutch++ split (blocks with n s^2 >= 2e7):
+"""The fixed-point products of the Hutch++ split (blocks with
+n s^2 >= 2e7, FP32 2e8):
 orth against an extended-precision QR at the edges of its tiles and row chunks, blocks
 that leave the fixed-point range (heavy rows, infinities), dropped columns,
 strides, and the projection through whole solves against the oracle.
@@ -62,7 +63,9 @@ def _run(y, pad=0, in_place=False):
 @pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
 @pytest.mark.parametrize("n,s,pad,in_place", [
     (4883, 64, 0, False), (5121, 63, 1, True), (33000, 25, 3, False), (50000, 20, 0, True),
-    (55001, 20, 20, False), (200129, 10, 2, True), (408231, 7, 1, False), (2300003, 3, 0, False)])
+    (55001, 20, 20, False), (200129, 10, 2, True), (408231, 7, 1, False), (2300003, 3, 0, False),
+    (12289, 64, 0, False), (49001, 64, 2, True), (50401, 63, 1, False), (80003, 25, 0, True),
+    (500009, 20, 20, False), (502001, 10, 2, True), (2000003, 10, 0, False), (1040001, 7, 0, True)])
 def test_orth_matches_qr(n, s, pad, in_place, dtype):
     y = _block(n, s, n + s, dtype)
     rank, a = _run(y, pad, in_place)
@@ -74,8 +77,8 @@ def test_orth_matches_qr(n, s, pad, in_place, dtype):
 
 @pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
 def test_orth_heavy_row_takes_the_general_products(dtype):
-    y = _block(60013, 20, 3, dtype)
-    y[31007] *= 3e2
+    y = _block(510013, 20, 3, dtype)
+    y[31007] *= 9e2
     rank, a = _run(y)
     tol = 2e-14 if dtype == torch.float64 else 1e-5
     assert rank == 20
@@ -83,7 +86,7 @@ def test_orth_heavy_row_takes_the_general_products(dtype):
 
 
 def test_orth_drops_a_dependent_and_a_zero_column():
-    y = _block(60013, 20, 4)
+    y = _block(130013, 20, 4)
     y[:, 7] = 0.5 * y[:, 2] - 3.0 * y[:, 5]
     y[:, 11] = 0.0
     rank, a = _run(y)
@@ -98,12 +101,12 @@ def test_orth_infinite_entry_ends_as_in_small_blocks():
         y[1234, 3] = float("inf")
         rank, a = _run(y)
         return rank, np.isfinite(a).all(axis=0).tolist()
-    assert parts(60013) == parts(40013)  # (the smaller block is below the fixed-point sizes)
+    assert parts(130013) == parts(40013)  # (the smaller block is below the fixed-point sizes)
 
 
 @pytest.mark.parametrize("probes,gaussian", [(60, 0), (61, 0), (60, 1)])
 def test_split_in_solves_matches_oracle(probes, gaussian):
-    A = W.laplacian_2d(241, 210, shift=0.5)
+    A = W.laplacian_2d(401, 320, shift=0.5)
     Q = A.to_scipy()
     with B.Handle.from_csr(A) as h:
         got = h.oslq(probes, 6, seed=3, gaussian=gaussian)
