@@ -712,8 +712,8 @@ __device__ double tridiag_gauss_log(double* d, double* e, double* z, int S, int 
 // three FP64 operations a step (t_i + s is not rounded: over random SPD T the
 // error against extended precision is 5.5e-16 root mean square, 7.1e-16 by the
 // continued fraction) and one division at the end, where the continued
-// fraction is a chain of m divisions (30 steps: 34 -> 14 us a launch with two
-// operations a step, which round t_i + s; the FP64 pipe issues an operation in
+// fraction is a chain of m divisions (30 steps: 34 -> 14 us a launch, with two
+// operations a step as with three; the FP64 pipe issues an operation in
 // 64 clocks); every kQuadRescale steps the
 // pair is scaled by a power of two (a step changes its size by at most
 // (1 + s) 4 and at least lambda_min).  One CTA per probe, one node per
