@@ -636,9 +636,10 @@ int launch_spmm_fix(const SpmmBatch<double>& b, cudaStream_t s) {
   if (dim == 3 ? ndc != 7 : (ndc != 5 && ndc != 13)) ndc = 0;
   for (int j = 0; j < b.njobs; ++j)  // (compiled counts: the middle entry is the diagonal)
     if (ndc && b.jobs[j].dinfo.off[ndc / 2] != 0) ndc = 0;
-  // Test hook: see launch_spmm_dia.
+  // Test hook: see launch_spmm_dia; "sketch" stalls the products without dots
+  // alone (the sketch's).
   const char* stall_env = getenv("LOGDET_TEST_SWEEP_STALL");
-  const bool stall = stall_env && stall_env[0] == '1';
+  const bool stall = stall_env && (stall_env[0] == '1' || (nd == 0 && !strcmp(stall_env, "sketch")));
   const unsigned extra_tx = stall ? 16u : 0u;
   const unsigned long long wait_ns = stall ? 20000000ull : kDiaWaitNs;
   const int grid = std::max(1, std::min(b.total_tiles, 2 * sm_count()));
@@ -672,7 +673,7 @@ int launch_spmm_fix(const SpmmBatch<double>& b, cudaStream_t s) {
 }
 
 int fix_spmm_block(const logdet_ctx* h, const int2* fix, int ka, const double* x, double* y, int ld,
-                   int xexp, cudaStream_t st) {
+                   int xexp, int* err_host, cudaStream_t st) {
   DevBuf<int> flags(st);
   LD_TRY(flags.alloc(2));
   LD_TRY(flags.zero());
@@ -693,7 +694,9 @@ int fix_spmm_block(const logdet_ctx* h, const int2* fix, int ka, const double* x
   J.xexp = xexp;
   LD_TRY(fix_job(J, h, g, fix, ka, flags.p));
   B.tile_start[1] = B.total_tiles = J.ntiles;
-  return launch_spmm_fix(B, st);
+  LD_TRY(launch_spmm_fix(B, st));
+  LD_CUDA(cudaMemcpyAsync(err_host, flags.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+  return LOGDET_OK;
 }
 
 }  // namespace ld

@@ -37,9 +37,10 @@ int fix_values(const logdet_ctx* h, double c, double shift, int ka, int2* out, c
 int fix_job(SpmmJob<double>& J, const logdet_ctx* h, const FixGeom& g, const int2* fix, int ka,
             int* bad);
 // One product y = A x over a block whose entries are below 2^xexp in
-// magnitude (no dots).
+// magnitude (no dots).  *err_host (pinned) is written in stream order: nonzero
+// if a staged copy's wait gave up, and y is not complete then.
 int fix_spmm_block(const logdet_ctx* h, const int2* fix, int ka, const double* x, double* y, int ld,
-                   int xexp, cudaStream_t st);
+                   int xexp, int* err_host, cudaStream_t st);
 // Batched launch (all jobs with fix != nullptr and one grid dimension).
 int launch_spmm_fix(const SpmmBatch<double>& b, cudaStream_t s);
 

@@ -662,7 +662,7 @@ struct Solve : ISolve {
   double *h_out = nullptr, *h_edot = nullptr;
   int *h_meff = nullptr, *h_keep = nullptr;
   uint32_t *h_status = nullptr, *h_status1 = nullptr;
-  int* h_err = nullptr;  // [2]: a diagonal-path wait gave up (phase 1, last run)
+  int* h_err = nullptr;  // [2]: a diagonal-path wait gave up (phase 1 or the sketch product, last run)
   cudaEvent_t ev_done = nullptr;
   const uint64_t* dev_keys = nullptr;  // graph plans: probe keys in device memory
   // Group member (solve_shifts): the Krylov phases run in one wide run over
@@ -1100,7 +1100,7 @@ struct Solve : ISolve {
   // (below 9 from 53-bit uniforms).
   int sketch_fix(const T* S, T* Y) {
     if constexpr (std::is_same<T, double>::value)
-      return fix_spmm_block(h, fixv.p, fix_ka, S, Y, lds, 4, st);
+      return fix_spmm_block(h, fixv.p, fix_ka, S, Y, lds, 4, h_err, st);
     else
       return LOGDET_EINVAL;
   }
