@@ -38,6 +38,13 @@ struct DiaInfo {
 };
 
 
+// Largest dynamic shared memory of a kernel without static shared memory.  The
+// limit that cudaFuncSetAttribute sets belongs to the kernel, for every thread
+// of the process: each launch site sets a bound over all its launches' sizes,
+// never its own size, which could be below what another thread is about to
+// launch with.
+constexpr int kMaxDynSmem = 227 * 1024;
+
 // ---------------------------------------------------------------------------
 // Errors.  Every host function returns an int code; the detail text of the
 // calling thread's last failure is kept in a thread-local string.

@@ -301,7 +301,7 @@ static int orth_t(int n, int s, const TY* Y, int ldy, TY* A, int lda, double* ws
   const size_t apply_smem = sizeof(TY) * ((size_t)s * s + 32 * (size_t)(s | 1));
   if (apply_smem > 48 * 1024)
     LD_CUDA(cudaFuncSetAttribute(k_apply_rinv<TY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)apply_smem));
+                                 kMaxDynSmem));
   for (int round = 0; round < 2; ++round) {
     ProfScope prof(KC_QR, st, 2.0 * n * (double)s * s * 2.0, 2.0 * sizeof(TY) * n * s);
     prof_count();
@@ -1253,7 +1253,7 @@ int hessenberg_log_e1(const double* H, int ldh, const int* msteps, int m, int np
   const size_t smem = smem_mats * mat;
   const int threads = kLogThreads;
   if (smem > 48 * 1024)
-    LD_CUDA(cudaFuncSetAttribute(k_hesslog, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LD_CUDA(cudaFuncSetAttribute(k_hesslog, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   ProfScope prof(KC_SMALL, st);
   k_hesslog<<<nprobe, threads, smem, st>>>(H, ldh, msteps, m, c, ldc, ws, status, gl, smem_mats);
   LD_CHECK_LAUNCH();

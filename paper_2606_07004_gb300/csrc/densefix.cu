@@ -51,8 +51,12 @@ constexpr int kSumBits = 28;     // H of the sums over rows
 constexpr int kAppBits = 30;     // H of the applies
 constexpr int kAtgBits = 24;     // A^T G: entries as 24 + 32-bit integers
 constexpr int kSlotRowsMax = 16384;           // 2^14 rows of 2^48 units: below 2^63
+// Shared memory over all shapes (launch limits): sums (staged chunks of at most
+// 2048 column slots, 8 bytes and A^T G's 4) and applies (64 columns).
+constexpr int kSumsSmem = 16 * kFT * 8 + 2 * 2048 * (8 + 4);
 constexpr int kAppRows = 128;                 // rows of an apply's chunk: four a lane
 constexpr int kAppStride = kAppRows + 2;      // staged column stride: 16-byte steps, banks spread
+constexpr int kAppSmem = kMaxSketch * kMaxSketch * 8 + 2 * kMaxSketch * kAppStride * 8;
 
 // Elements of 2^f > |x| from the bits: the exponent of one above it.
 __device__ __forceinline__ unsigned abs_word(double x) { return __double2hiint(x) & 0x7fffffff; }
@@ -532,7 +536,7 @@ int sums_fix(const TY* Y, int ldy, int n, int s, int r, uint64_t key, const uint
   const int chunk = RS * std::max(1, std::min(32, 2048 / (RS * wide)));
   const size_t smem = 16 * kFT * 8 + 2 * (size_t)chunk * 4 * s4 * 8 + (ATG ? 2 * (size_t)chunk * 4 * r4 * 4 : 0);
   auto kern = k_sums_fix<TY, ATG>;
-  LD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  LD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSumsSmem));
   const int nslots = densefix_slots(n);
   kern<<<std::min(nslots, resident(kern, kFT, smem)), kFT, smem, st>>>(
       Y, ldy, n, s, r, key, keyp, c.exp, c.bad, slot_rows(n), nslots, RS, chunk, part);
@@ -546,7 +550,7 @@ int apply_launch(const double* Y, int ldy, int n, int s, int r, const double* Rm
   const int r4 = div_up(r, 4), threads = 32 * r4;
   const size_t smem = (size_t)s * 4 * r4 * 8 + 2 * (size_t)s * kAppStride * 8;
   auto kern = k_apply_fix<PROJ>;
-  LD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  LD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kAppSmem));
   kern<<<std::min(div_up(n, kAppRows), resident(kern, threads, smem)), threads, smem, st>>>(
       Y, ldy, n, s, r, Rm, c.exp, c.bad, key, keyp, A, lda);
   LD_CHECK_LAUNCH();

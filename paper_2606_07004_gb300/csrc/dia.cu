@@ -911,7 +911,7 @@ int launch_spmm_dia(const SpmmBatch<float>& b, int threads, cudaStream_t s) {
     const int nr = 2 * amax + 1 + kSweepPrefetch;                                            \
     const size_t smem = sweep_smem_bytes(nr, slot_floats, threads);                          \
     if (smem > 48 * 1024)                                                                    \
-      LD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
+      LD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem)); \
     int per_sm = 0;                                                                          \
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);             \
     if (per_sm < 1) per_sm = 1;                                                              \

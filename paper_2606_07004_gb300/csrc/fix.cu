@@ -651,7 +651,7 @@ int launch_spmm_fix(const SpmmBatch<double>& b, cudaStream_t s) {
                          : ndc == 13 ? k_spmm_fix<NO, SELF, 13, 2>                             \
                          : ndc == 5  ? k_spmm_fix<NO, SELF, 5, 2>                              \
                                      : k_spmm_fix<NO, SELF, 0, 2>;                             \
-    LD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));    \
+    LD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kFixSmem)); \
     kern<<<grid, kFixThreads, smem, s>>>(b, extra_tx, wait_ns);                                \
     break;                                                                                     \
   }

@@ -292,7 +292,7 @@ int grid_apply(const logdet_ctx* h, const typename Compute<T>::type* tab, const 
   const size_t smem = grid_smem_bytes(R, sizeof(CT));
   if (smem > 48 * 1024)
     LD_CUDA(cudaFuncSetAttribute(k_grid_apply<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem));
+                                 kMaxDynSmem));
   const int nseg = div_up(h->gx, kGridTX * kGridP);
   const int nchunk = ld / V;
   const long long items = (long long)div_up(h->gy, kGridTY) * nseg * nchunk;
