@@ -640,6 +640,20 @@ struct PinnedHost {
   ~PinnedHost() { pinned_release(p, cap, st); }
 };
 
+// FP64 blocks of a grid stencil (widths ld and, of the sketch, lds), above
+// kFixMinBlock: pass 1 in fixed point.
+static bool fix_applies(const logdet_ctx* h, const SolveCfg& c, int ld, int lds) {
+  if (h->kind != 0 || (size_t)h->n * std::min(ld, lds) * sizeof(double) <= kFixMinBlock ||
+      !fix_balanced(h, c.shift))
+    return false;
+  FixGeom g;
+  for (int w : {ld, lds}) {
+    if (!fix_geom(h, w, w, &g)) return false;
+    if (c.block_width > 0 && !fix_geom(h, std::min(c.block_width, w), w, &g)) return false;
+  }
+  return true;
+}
+
 template <typename T>
 struct Solve : ISolve {
   logdet_ctx* h;
@@ -890,19 +904,10 @@ struct Solve : ISolve {
   }
 
   double cscale() const { return c.method == 0 ? alpha : gamma; }
-  // FP64 blocks of a grid stencil, above kFixMinBlock: pass 1 in fixed point
   // (group members share one run whose columns have factors of their own, and
-  // keep the CSR pass).
+  // keep the CSR pass)
   bool use_fix() const {
-    if (!std::is_same<T, double>::value || grouped || h->kind != 0) return false;
-    const int narrow = s ? std::min(ld, lds) : ld;
-    if ((size_t)n * narrow * sizeof(double) <= kFixMinBlock || !fix_balanced(h, c.shift)) return false;
-    FixGeom g;
-    for (int w : {ld, s ? lds : ld}) {
-      if (!fix_geom(h, w, w, &g)) return false;
-      if (c.block_width > 0 && !fix_geom(h, std::min(c.block_width, w), w, &g)) return false;
-    }
-    return true;
+    return std::is_same<T, double>::value && !grouped && fix_applies(h, c, ld, s ? lds : ld);
   }
   // Group member: free the start block once the group has copied it.
   void release_start() {
@@ -1310,10 +1315,13 @@ size_t estimate_solve_bytes(const logdet_ctx* h, const SolveCfg& c) {
   const int s = c.plain ? 0 : c.P / 3, r = c.plain ? c.P : c.P - 2 * s, b = s + r;
   const size_t ld = round_up(b, vec), lds = std::max(round_up(s, vec), vec);
   const int m = c.m, k = c.method == 0 ? 2 : std::min(c.k, c.m);
-  // Scaled values, plus (FP32 blocks of a grid stencil) the values per row
-  // and diagonal of the sweep paths.
+  // Scaled values (FP64 in fixed point: per row and diagonal in their place),
+  // plus (FP32 blocks of a grid stencil) the values per row and diagonal of the
+  // sweep paths.
+  const bool fix_vals = !f32 && fix_applies(h, c, (int)ld, s ? (int)lds : (int)ld);
+  const size_t entries = std::max((size_t)h->nnz, fix_vals ? (size_t)h->dia.ndiag * n : 0);
   const bool sweep_vals = f32 && !b16 && !df && h->kind == 0 && h->dia.ndiag > 0 && h->dia_slot;
-  const size_t vals = (h->kind == 1 ? grid_table_count(h) * 8 : (size_t)h->nnz * (f32 ? 4 : 8)) +
+  const size_t vals = (h->kind == 1 ? grid_table_count(h) * 8 : entries * (f32 ? 4 : 8)) +
                       (sweep_vals ? (size_t)dia_pad(h->dia.ndiag) * n * 4 : 0);
   const TileGeom g = tile_geom((int)ld, vec, 0, 0, (int)n);
   const size_t ntiles = div_up((int)n, g.tile_rows);
