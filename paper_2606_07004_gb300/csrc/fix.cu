@@ -17,8 +17,8 @@
 // below that of an FP64 sum, which rounds every product and addition to 2^-53
 // of its size; measured against 64-bit references the estimates' errors are
 // unchanged (3e-16 to 1e-15).  An entry of x too large for its column's F (or not finite) sets
-// a flag, and k_spmm_fix_general, launched after every product, then redoes
-// it with FP64 arithmetic.
+// the job's flag; k_spmm_fix_general, launched after every product, then redoes
+// it with FP64 arithmetic, and takes the job's later products alone.
 //
 // x arrives as in the FP32 sweeps (dia.cu): a CTA sweeps a segment of a line
 // (2D) or a tile of a plane (3D) over consecutive lines or planes, keeping
@@ -56,6 +56,7 @@ constexpr int kFixThreads = 256;
 constexpr int kFixSmem = 112 * 1024;           // per CTA
 constexpr int kFixValRegs = 4;                 // values a thread loads ahead
 constexpr int kFixPoints = 4;                  // points of a line or plane a thread takes
+constexpr int kFixMaxWindows = 15;              // ring slots: a barrier each, in 128 bytes with `skip`
 constexpr int kFixAhead = 1;                    // windows loaded ahead of the current line's
 constexpr int kFixMaxWidth = 128;              // TMA box: 256 words
 
@@ -84,8 +85,13 @@ __host__ __device__ inline FixSmem fix_smem(const DiaInfo& d, int T, int tx, int
 struct FixUnit {
   int gu, jb, seg0, segT, k0, nl;  // as SwUnit in dia.cu
 };
-template <int DIM>
-__device__ __forceinline__ void fix_unit(FixUnit& U, const SpmmBatch<double>& B, int gu) {
+// Unit gu; with SKIP, the CTA's first one from gu on whose job is not in *skip.
+template <int DIM, bool SKIP>
+__device__ __forceinline__ void fix_unit(FixUnit& U, const SpmmBatch<double>& B, int gu,
+                                         const volatile unsigned* skip) {
+  static_assert(kMaxJobs <= 32, "one bit a job");
+  if constexpr (SKIP)
+    while (gu < B.total_tiles && (*skip >> find_job(B, gu) & 1u)) gu += gridDim.x;
   U.gu = gu;
   if (gu >= B.total_tiles) return;
   U.jb = find_job(B, gu);
@@ -103,6 +109,12 @@ __device__ __forceinline__ void fix_unit(FixUnit& U, const SpmmBatch<double>& B,
   }
   U.k0 = chunk * J.dia_kc;
   U.nl = min(J.dia_kc, J.dia_nlines - U.k0);
+}
+
+// One warp: the jobs whose flag is set, a bit each.
+__device__ __forceinline__ unsigned jobs_out_of_range(const SpmmBatch<double>& B) {
+  const int j = threadIdx.x & 31;
+  return __ballot_sync(~0u, j < B.njobs && __ldcg(B.jobs[j].bad) != 0);
 }
 
 // Row of point p of a unit's line or plane k, or -1 outside the grid.
@@ -166,7 +178,13 @@ __device__ __forceinline__ int fix_exp(const SpmmJob<double>& J, int p) {
 // summed in integers from the window's converted x and the unrounded y:
 // about 11 instructions against a load and a 64-clock DFMA (window-4 solve:
 // 98 -> 84 ms with the conversion above; a single dot: unchanged).
-template <int NOTH, bool SELF, int NDC, int DIM>
+// MANY: several jobs a launch.  Jobs whose flag is set already are the general
+// kernel's alone (their vectors have left the range, mostly for good): a lone
+// one ends the launch at once, of several the units are skipped.  Either reads
+// the flags once for the whole CTA, since another CTA may be setting one.  (The
+// skipping cost a lone 128^3 single-dot pass 1 to 2 %, through the compiler's
+// schedule of the sums: 683 us against 695.)
+template <int NOTH, bool SELF, int NDC, int DIM, bool MANY>
 __global__ void __launch_bounds__(kFixThreads, 2)
     k_spmm_fix(const __grid_constant__ SpmmBatch<double> B, unsigned extra_tx,
                unsigned long long wait_ns) {
@@ -175,8 +193,19 @@ __global__ void __launch_bounds__(kFixThreads, 2)
   constexpr bool kEarly = NOTH <= 3;  // window vectors loaded before the sums
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const uint32_t bar0 = smem_addr(smem_raw);
+  int* xo_tab = reinterpret_cast<int*>(smem_raw + 128);
+  volatile unsigned* skip = reinterpret_cast<unsigned*>(smem_raw + 8 * kFixMaxWindows);
+  if constexpr (MANY) {
+    if (threadIdx.x < 32) {
+      const unsigned out = jobs_out_of_range(B);
+      if (threadIdx.x == 0) *skip = out;
+    }
+    __syncthreads();
+  } else {
+    if (__syncthreads_or(threadIdx.x == 0 && __ldcg(B.jobs[0].bad))) return;
+  }
   FixUnit C;
-  fix_unit<DIM>(C, B, blockIdx.x);
+  fix_unit<DIM, MANY>(C, B, blockIdx.x, skip);
   if (C.gu >= B.total_tiles) return;
   // Every job of a launch has the same matrix structure constants up to its
   // sizes; the ring is laid out per job, so a CTA drains before it changes.
@@ -188,9 +217,8 @@ __global__ void __launch_bounds__(kFixThreads, 2)
   int G = 1, R = 1, r = 0, g = 0, nd = 0, width = 0, A = 0, col0 = 0, ldy = 0, noth = 0, dself = 0;
   int K[V], ex[V], rmin = 1 << 20;
   bool live = false;
-  int* xo_tab = reinterpret_cast<int*>(smem_raw + 128);
   if (threadIdx.x == 0) {
-    for (int q = 0; q < 16; ++q) mbar_init(bar0 + 8 * q, 1);
+    for (int q = 0; q < kFixMaxWindows; ++q) mbar_init(bar0 + 8 * q, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -210,7 +238,7 @@ __global__ void __launch_bounds__(kFixThreads, 2)
       ++issued;
       if (++pslot == nr) pslot = 0;
       if (++pq == P.nl + 2 * J.dinfo.A) {
-        fix_unit<DIM>(P, B, P.gu + gridDim.x);
+        fix_unit<DIM, MANY>(P, B, P.gu + gridDim.x, skip);
         pq = 0;
       }
     }
@@ -445,54 +473,90 @@ __global__ void __launch_bounds__(kFixThreads, 2)
     if (rslot >= nr) rslot -= nr;
     t0 += nwin;
     produce(t0);
-    fix_unit<DIM>(C, B, C.gu + gridDim.x);
+    fix_unit<DIM, MANY>(C, B, C.gu + gridDim.x, skip);
   }
 }
 
+// A 2^(ka - 60), A = a.x 2^30 + a.y, in FP64: leading one, shift and rounding
+// in integers, where the conversion and its scaling would take the FP64 pipe as
+// long as the entry's two multiply-adds.
+__device__ __forceinline__ double fix_entry(int2 a, int ka) {
+  const long long A = ((long long)a.x << 30) + a.y;
+  if (A == 0) return 0.0;
+  const unsigned long long m = A < 0 ? -(unsigned long long)A : (unsigned long long)A;
+  const int lz = __clzll((long long)m);
+  const unsigned long long f = m << lz;
+  const unsigned long long r = (f >> 11) + ((f >> 10) & 1);  // 2^52 <= r <= 2^53
+  const long long bits = ((long long)(1025 + ka - lz) << 52) + (long long)r;
+  return __longlong_as_double(A < 0 ? bits | (1LL << 63) : bits);
+}
+
 // The same product, y and partials with FP64 arithmetic, for jobs whose flag
-// is set (x outside its column's range); a few reads otherwise.
-template <int DIM>
-__global__ void __launch_bounds__(kFixThreads)
+// is set (x outside its column's range); a read of the flag otherwise.  ND:
+// bound of the jobs' dots (their sums stay in registers).  The FP64 pipe
+// bounds it like the CSR pass: 64 x 63 x 61 Laplacian with one entry raised by
+// 8, 60 probes, 30 steps, all but the first few beyond the range, the SpMM
+// passes of a solve 5.9 ms (CSR pass 6.1), window 4 11.7 (12.9); 15.1 and 30.2
+// with the dots' sums in local memory, the conversions on the FP64 pipe and the
+// fixed-point pass run as well in every step.
+template <int ND, int DIM>
+__global__ void __launch_bounds__(kFixThreads, ND > 4 ? 2 : ND > 2 ? 3 : 4)
     k_spmm_fix_general(const __grid_constant__ SpmmBatch<double> B) {
   __shared__ AccD red[kFixThreads * 2];
-  for (int gu = blockIdx.x; gu < B.total_tiles; gu += gridDim.x) {
-    FixUnit U;
-    fix_unit<DIM>(U, B, gu);
+  const unsigned in_range = ~jobs_out_of_range(B);
+  if (in_range == ~0u) return;
+  FixUnit U;
+  for (fix_unit<DIM, true>(U, B, blockIdx.x, &in_range); U.gu < B.total_tiles;
+       fix_unit<DIM, true>(U, B, U.gu + gridDim.x, &in_range)) {
     const SpmmJob<double>& J = B.jobs[U.jb];
-    if (!__ldcg(J.bad)) continue;
     const DiaInfo& D = J.dinfo;
     const int nd = D.ndiag, G = J.width / 2, R = kFixThreads / G;
     const int r = threadIdx.x / G, g = threadIdx.x - r * G, col0 = J.col_off + g * 2;
     const bool live = r < R;
-    const double scale = ldexp(1.0, J.ka - 60);
-    AccD acc[kMaxWin][2];
-    for (int d = 0; d < kMaxWin; ++d) acc[d][0].zero(), acc[d][1].zero();
+    AccD acc[ND > 0 ? ND : 1][2];
+#pragma unroll
+    for (int d = 0; d < ND; ++d) acc[d][0].zero(), acc[d][1].zero();
     for (int k = U.k0; live && k < U.k0 + U.nl; ++k)
       for (int p = r; p < J.dia_T; p += R) {
         const int row = fix_row<DIM>(J, U, k, p);
         if (row < 0) continue;
+        const int2* fa = J.fix + (size_t)row * nd;
         double s0 = 0.0, s1 = 0.0;
-        for (int d = 0; d < nd; ++d) {
-          const int2 a = __ldg(J.fix + (size_t)row * nd + d);
-          if (a.x == 0 && a.y == 0) continue;  // no entry: the neighbour may not exist
-          const double av = fma((double)a.x, 0x1p30, (double)a.y) * scale;
-          const double2 x = __ldg(reinterpret_cast<const double2*>(
-              J.x + (size_t)(row + D.off[d]) * J.ld + col0));
-          s0 = fma(av, x.x, s0);
-          s1 = fma(av, x.y, s1);
+        for (int d0 = 0; d0 < nd; d0 += 4) {
+          int2 a[4];
+          double2 x[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) a[q] = d0 + q < nd ? __ldg(fa + d0 + q) : make_int2(0, 0);
+#pragma unroll
+          for (int q = 0; q < 4; ++q)  // (no entry: the neighbour may not exist)
+            x[q] = a[q].x | a[q].y ? __ldg(reinterpret_cast<const double2*>(
+                                         J.x + (size_t)(row + D.off[d0 + q]) * J.ld + col0))
+                                   : make_double2(0.0, 0.0);
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (d0 + q < nd) {
+              const double av = fix_entry(a[q], J.ka);
+              s0 = fma(av, x[q].x, s0);
+              s1 = fma(av, x[q].y, s1);
+            }
         }
         const size_t off = (size_t)row * J.ld + col0;
         *reinterpret_cast<double2*>(J.y + off) = make_double2(s0, s1);
-        for (int d = 0; d < J.ndots; ++d) {
-          const double2 u = __ldg(reinterpret_cast<const double2*>(J.dotv[d] + off));
-          acc[d][0].fma(u.x, s0);
-          acc[d][1].fma(u.y, s1);
+#pragma unroll
+        for (int d = 0; d < ND; ++d) {
+          if (d < J.ndots) {
+            const double2 u = __ldg(reinterpret_cast<const double2*>(J.dotv[d] + off));
+            acc[d][0].fma(u.x, s0);
+            acc[d][1].fma(u.y, s1);
+          }
         }
       }
-    for (int d = 0; d < J.ndots; ++d)
-      cta_reduce_write<double, AccD>(red, acc[d], live, G, R, J.col_off, J.width,
-                                     J.part + (size_t)d * J.ld * J.ntiles, J.ntiles,
-                                     gu - B.tile_start[U.jb]);
+#pragma unroll
+    for (int d = 0; d < ND; ++d)
+      if (d < J.ndots)
+        cta_reduce_write<double, AccD>(red, acc[d], live, G, R, J.col_off, J.width,
+                                       J.part + (size_t)d * J.ld * J.ntiles, J.ntiles,
+                                       U.gu - B.tile_start[U.jb]);
     __syncthreads();
   }
 }
@@ -516,7 +580,7 @@ __global__ void k_fix_values(const int* __restrict__ rowptr, const int* __restri
 bool fix_geom(const logdet_ctx* h, int width, int ld, FixGeom* out) {
   const DiaInfo& d = h->dia;
   if (h->kind != 0 || d.ndiag == 0 || !h->dia_slot || width % 2 || width < 2 || width > kFixMaxWidth ||
-      2 * d.A + 1 + kFixAhead > 16 || (d.dim == 3 && (long long)d.P * ld >= (1LL << 30)))
+      2 * d.A + 1 + kFixAhead > kFixMaxWindows || (d.dim == 3 && (long long)d.P * ld >= (1LL << 30)))
     return false;
   const int R = kFixThreads / (width / 2);
   FixGeom g;
@@ -585,14 +649,14 @@ int fix_values(const logdet_ctx* h, double c, double shift, int ka, int2* out, c
 }
 
 int fix_job(SpmmJob<double>& J, const logdet_ctx* h, const FixGeom& g, const int2* fix, int ka,
-            int* flags) {
+            int* err, int* bad) {
   const DiaInfo& d = h->dia;
   J.dinfo = d;
   J.fix = fix;
   J.ka = ka;
   J.hn = std::ilogb((double)J.n) / 2;
-  J.err = flags;
-  J.bad = flags + 1;
+  J.err = err;
+  J.bad = bad;
   J.dia_T = g.T;
   J.dia_kc = g.kc;
   J.dia_nseg = g.nseg;
@@ -645,12 +709,14 @@ int launch_spmm_fix(const SpmmBatch<double>& b, cudaStream_t s) {
   const int grid = std::max(1, std::min(b.total_tiles, 2 * sm_count()));
   {
     ProfScope prof(KC_SPMM, s, flops, bytes);
+#define LD_FIX_KERN(NO, SELF, NC, DM) \
+  (b.njobs > 1 ? k_spmm_fix<NO, SELF, NC, DM, true> : k_spmm_fix<NO, SELF, NC, DM, false>)
 #define LD_FIX_CASE(NO, SELF)                                                                  \
   {                                                                                            \
-    auto kern = dim == 3 ? (ndc == 7 ? k_spmm_fix<NO, SELF, 7, 3> : k_spmm_fix<NO, SELF, 0, 3>) \
-                         : ndc == 13 ? k_spmm_fix<NO, SELF, 13, 2>                             \
-                         : ndc == 5  ? k_spmm_fix<NO, SELF, 5, 2>                              \
-                                     : k_spmm_fix<NO, SELF, 0, 2>;                             \
+    auto kern = dim == 3 ? (ndc == 7 ? LD_FIX_KERN(NO, SELF, 7, 3) : LD_FIX_KERN(NO, SELF, 0, 3)) \
+                         : ndc == 13 ? LD_FIX_KERN(NO, SELF, 13, 2)                            \
+                         : ndc == 5  ? LD_FIX_KERN(NO, SELF, 5, 2)                             \
+                                     : LD_FIX_KERN(NO, SELF, 0, 2);                            \
     LD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kFixSmem)); \
     kern<<<grid, kFixThreads, smem, s>>>(b, extra_tx, wait_ns);                                \
     break;                                                                                     \
@@ -663,11 +729,26 @@ int launch_spmm_fix(const SpmmBatch<double>& b, cudaStream_t s) {
       LD_FIX_CASE(kMaxWin - 1, true)
     } while (0);
 #undef LD_FIX_CASE
+#undef LD_FIX_KERN
     LD_CHECK_LAUNCH();
   }
+  // Four CTAs per SM: the FP64 pipe is full from two.
+  const int ggrid = std::max(1, std::min(b.total_tiles, 4 * sm_count()));
   ProfScope prof(KC_SPMM, s);
-  if (dim == 3) k_spmm_fix_general<3><<<grid, kFixThreads, 0, s>>>(b);
-  else k_spmm_fix_general<2><<<grid, kFixThreads, 0, s>>>(b);
+#define LD_FIX_GENERAL(ND)                                                       \
+  {                                                                              \
+    if (dim == 3) k_spmm_fix_general<ND, 3><<<ggrid, kFixThreads, 0, s>>>(b);    \
+    else k_spmm_fix_general<ND, 2><<<ggrid, kFixThreads, 0, s>>>(b);             \
+    break;                                                                       \
+  }
+  do {
+    if (nd == 0) LD_FIX_GENERAL(0)
+    if (nd == 1) LD_FIX_GENERAL(1)
+    if (nd == 2) LD_FIX_GENERAL(2)
+    if (nd <= 4) LD_FIX_GENERAL(4)
+    LD_FIX_GENERAL(kMaxWin)
+  } while (0);
+#undef LD_FIX_GENERAL
   LD_CHECK_LAUNCH();
   return LOGDET_OK;
 }
@@ -692,7 +773,7 @@ int fix_spmm_block(const logdet_ctx* h, const int2* fix, int ka, const double* x
   J.ld = J.width = J.b = ld;
   J.nnz = h->nnz;
   J.xexp = xexp;
-  LD_TRY(fix_job(J, h, g, fix, ka, flags.p));
+  LD_TRY(fix_job(J, h, g, fix, ka, flags.p, flags.p + 1));
   B.tile_start[1] = B.total_tiles = J.ntiles;
   LD_TRY(launch_spmm_fix(B, st));
   LD_CUDA(cudaMemcpyAsync(err_host, flags.p, sizeof(int), cudaMemcpyDeviceToHost, st));

@@ -32,10 +32,12 @@ inline bool fix_balanced(const logdet_ctx* h, double shift) {
 int fix_scale(const logdet_ctx* h, double c, double shift);
 int fix_values(const logdet_ctx* h, double c, double shift, int ka, int2* out, cudaStream_t st);
 
-// A job's fixed-point fields (fix, ka, hn, bad) and tensor map from its x,
-// ld, col_off and width; sig / sig_stride / xexp are the caller's.
+// A job's fixed-point fields (fix, ka, hn, err, bad) and tensor map from its x,
+// ld, col_off and width; sig / sig_stride / xexp are the caller's.  *bad is the
+// job's own: set when its columns leave the range, and from the next launch on
+// the fixed-point pass leaves the job to the general kernel.
 int fix_job(SpmmJob<double>& J, const logdet_ctx* h, const FixGeom& g, const int2* fix, int ka,
-            int* bad);
+            int* err, int* bad);
 // One product y = A x over a block whose entries are below 2^xexp in
 // magnitude (no dots).  *err_host (pinned) is written in stream order: nonzero
 // if a staged copy's wait gave up, and y is not complete then.

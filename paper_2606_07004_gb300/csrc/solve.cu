@@ -208,7 +208,7 @@ int KRun<T>::init(const int* rp, const int* ci, const typename ValOf<T>::type* v
   if (method != 0 && (size_t)2 * ld * ntiles * sizeof(Part) <= kNormPartMax)
     LD_TRY(npart.alloc((size_t)2 * ld * ntiles));
   if (diavals || fixvals) {
-    LD_TRY(dia_err.alloc(2));
+    LD_TRY(dia_err.alloc(1 + tune.split));
     LD_TRY(dia_err.zero());
   }
   LD_TRY(y.alloc(blk));
@@ -290,7 +290,7 @@ int KRun<T>::spmm_jobs(int j, std::vector<SpmmJob<T>>& out) const {
       if (sweep) {
         J.sig = ks.sig.p + j;
         J.sig_stride = m + 2;
-        LD_TRY(fix_job(J, hctx, fg, fixvals, fix_ka, dia_err.p));
+        LD_TRY(fix_job(J, hctx, fg, fixvals, fix_ka, dia_err.p, dia_err.p + 1 + q));
       }
     }
     out.push_back(J);

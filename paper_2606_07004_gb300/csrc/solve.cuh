@@ -111,7 +111,7 @@ struct KRun {
   const int2* fixvals = nullptr;   // fixed-point entries: the FP64 sweep (fix.cu), their scale
   int fix_ka = 0;
   FixGeom fg{};
-  DevBuf<int> dia_err;             // [0] set if a staged copy's wait gave up; [1] fixed-point range
+  DevBuf<int> dia_err;             // [0] set if a staged copy's wait gave up; [1 + slice] fixed-point range
   bool sweep = false;              // pass 1 runs the line sweep
   int sw_T = 0, sw_kc = 0, sw_nseg = 0, sw_nlines = 0, sw_tx = 0, sw_ty = 0, sw_txs = 0;
   int done_steps = 0;  // steps whose pass 1 has been issued
