@@ -5,52 +5,71 @@
 // measured), a 32 x 32 + 64-bit integer multiply-add 4.7, an FP32 one 1, so
 // n s^2 FP64 multiply-adds took the time (93 % FP64 pipe) of products that
 // read and write a few n s numbers.  A column is scaled by the power of two
-// 2^f above its largest entry and split into X = xh + 2^-32 xl, xh an integer
-// of H bits and xl the 32 bits that follow (signed, rounded to FP32's 24), and
+// 2^f above its largest entry and held as integers of 60 bits in two limbs.
 //
-//   X Y = xh yh + 2^-32 (xh yl + xl yh)    (+ 2^-64 xl yl, left out)
+// Sums over rows: X = xh + 2^-32 xl, xh an integer of H bits and xl the 32 bits
+// that follow (signed, rounded to FP32's 24), and
+//
+//   X Y = xh yh + 2^-32 (xh yl + xl yh)    (+ 2^-64 xl yl)
 //
 // takes one integer multiply-add, summed exactly, and two FP32 ones, whose sum
-// is H bits smaller.  A sum over rows (H = 28) thus carries rounding of
-// 2^-53 2^f and less a term, with random signs, where an FP64 sum also rounds
-// at every addition; a result of the applies (H = 30) is rounded to FP64 once.
-// That holds while 2^f is not far above a column's typical entry: beyond 64
-// times its mean magnitude (the entries of one heavy row, say), and for
-// infinities and NaN, the column flags the block and the FP64 kernels,
-// launched after each of these, run instead.
+// is H bits smaller and joins the integers every fourth row.  A^T G adds
+// 56-bit entries.  Applies: two limbs of 30 bits and three integer products.
+//
+// How exact: with a typical entry 2^f / rho (rho is about 10 for Gaussian
+// columns), Gram entries err by 1e-17 to 3e-17 on the diagonal and 3e-18 to
+// 1e-17 of the norms off it (NumPy replay against exact sums, rho = 8 to 16, n =
+// 4,883; FP64 sums 0.7e-16 to 1.6e-16 and 1e-17).  Orthonormal columns are off
+// the exact factor by 0.85e-16 to 1.03e-16 of their norm, by the FP64 kernels
+// 0.85e-16 to 0.92e-16 (rms; 13,007 and 24,001 x 64, 20,011 x 32, 50,021 x 20).  Blocks with
+// rho above 16 (the entries of one heavy row, say), infinities or NaN are
+// flagged, and the FP64 kernels, launched after each of these, run instead.
+// With FP32 cross terms in the applies too, and sums rounded at each fold,
+// columns were off by 1.1e-15 at rho = 8 and 1.3e-14 at 31 (4,883 x 64).
 //
 // FP32 blocks (mixed solves) take the two sums over rows as well, in place of
-// compensated FP32 dots of 17 operations.
+// compensated FP32 dots of 17 operations (which err by 2^-48): H = 28, cross
+// terms folded every 64th row, up to rho = 64.
 //
 // One GB300, us a launch before -> after (the FP64 or compensated FP32 kernel
 // against this one; column_scales adds 34 + 8 us at 1M x 20):
 //                            Y^T Y        Y R^-1       A^T G         G - A B
-//   1M x 20 FP64             415 -> 131   436 -> 163
-//   2.1M x 20 FP64           850 -> 265   911 -> 335   1689 -> 341   1531 -> 421
-//   1M x 40 FP32             610 -> 465                1174 -> 618
-// The integer multiply-adds' pipe bounds the sums (three of them a product, no
-// FP32 part: 200 us at 1M x 20, the pipe 81 % busy); the applies wait at the
-// chunk barrier as well.  The rule (densefix_ok), whole orthogonalisations:
-// FP64 125,000 x 20 (n s^2 = 5e7) 408 -> 224 us, 1M x 10 740 -> 413; FP32
-// 500,000 x 20 (2e8) 430 -> 362 us, but a server's burst of blocks of 1e8 and
-// less, whose launches count (three more a sum), took 28.9 ms with the
-// fixed-point sums and 28.7 without.
+//   1M x 20 FP64             415 -> 150   436 -> 242
+//   2.1M x 20 FP64           850 -> 303   911 -> 500   1689 -> 341   1531 -> 652
+//   1M x 40 FP32             610 -> 445                1174 -> 626
+// The integer multiply-adds' pipe bounds the applies (with FP32 cross terms 163,
+// 335 and 421 us), it and the conversions of the cross terms the sums (131 us
+// with those once in 64 rows).
 #include "densefix.cuh"
 #include "dense.cuh"
 #include "krylov.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace ld {
 
 namespace {
 
 constexpr int kFT = 256;         // threads of the sums over rows
-constexpr int kFoldRows = 64;    // rows a thread sums before it folds: 64 2^56 = 2^62
-constexpr int kSumBits = 28;     // H of the sums over rows
-constexpr int kAppBits = 30;     // H of the applies
+// Gram sums: H, the rows a thread sums before it folds (2^62 at most) and those
+// whose FP32 cross terms it sums (below 2^31 units).  An FP32 block's entries
+// have 24 bits, and the compensated sums before erred by 2^-48.
+template <typename TY> struct Gram;
+template <> struct Gram<double> { static constexpr int kBits = 29, kFold = 16, kCross = 4; };
+template <> struct Gram<float> { static constexpr int kBits = 28, kFold = 64, kCross = 64; };
+constexpr int kAtgFold = 64;     // A^T G: 64 2^56 = 2^62
+// 2^f above this many times a column's mean magnitude flags the block.  (Gaussian
+// columns reach 12 at a million rows and 16 at 2^31.)
+template <typename TY> constexpr float max_over_mean() { return std::is_same<TY, double>::value ? 16.f : 64.f; }
 constexpr int kAtgBits = 24;     // A^T G: entries as 24 + 32-bit integers
-constexpr int kSlotRowsMax = 16384;           // 2^14 rows of 2^48 units: below 2^63
+constexpr int kSlotRowsMax = 16384;
+// Folded sums are kept in units of 2^fold_shift, so that a slot's stay below 2^62.
+inline int fold_shift(int rows_slot, int bits) {
+  int lg = 0;
+  while ((1 << lg) < rows_slot) ++lg;
+  return std::max(0, lg + bits - 62);
+}
 // Shared memory over all shapes (launch limits): sums (staged chunks of at most
 // 2048 column slots, 8 bytes and A^T G's 4) and applies (64 columns).
 constexpr int kSumsSmem = 16 * kFT * 8 + 2 * 2048 * (8 + 4);
@@ -102,6 +121,13 @@ __device__ __forceinline__ int2 to_limbs(TY x, int f) {
   const unsigned long long w = to_fixed<H>(x, f, m);
   const int lo = (int)(unsigned)w, hi = (int)(w >> 32) - (lo >> 31);
   return make_int2((hi ^ m) - m, __float_as_int((float)lo) ^ (m & 0x80000000));
+}
+// 30-bit limbs: X = xh 2^30 + xl below 2^60, 0 <= xl < 2^30 (rounded down).
+__device__ __forceinline__ int2 to_limbs30(double x, int f) {
+  int m;
+  const unsigned long long w = to_fixed<28>(x, f, m);
+  return make_int2((int)__funnelshift_r((unsigned)w, (unsigned)(w >> 32), 30) ^ m,
+                   ((int)(unsigned)w ^ m) & 0x3fffffff);
 }
 // v 2^ex (|ex| far from the exponent's limits).
 __device__ __forceinline__ double scaled(long long v, int ex) {
@@ -198,7 +224,7 @@ __global__ void __launch_bounds__(1024) k_col_exps(const unsigned* __restrict__ 
       const int f = m ? Bits<TY>::exp(m) : 0;
       // (a column outside FP32's range has an infinite or zero sum)
       const bool ok = m < Bits<TY>::kInf && (m == 0 || (f > -100 && f < 100 && a < 3e38f &&
-                                                        ldexpf(1.f, f) <= 64.f * (a / (float)n)));
+                                                        ldexpf(1.f, f) <= max_over_mean<TY>() * (a / (float)n)));
       ex[c] = ok ? f : 0;
       if (!ok) any = 1;
     }
@@ -221,17 +247,21 @@ __device__ __forceinline__ void unrank_tile(int q, int s, int& i, int& j) {
 // staged chunks, so that eight column loads feed 16 products; the
 // tiles times the row subsets fill the CTA.  A chunk is copied in while the
 // one before it is summed and converted in place by the threads that copied
-// it.  Sums are exact for kFoldRows rows, then go to shared memory in units of
-// 2^8 (below 2^-50 of the sum of 64 rows, with random signs).
+// it.  The integer sums are exact for Gram::kFold (kAtgFold) rows, then whole
+// units of 2^shift go to shared memory and the remainder stays, so that a slot
+// rounds once, at its end: by 2^-63 rows 2^2f at most.  The product xl yl is left
+// out but on the diagonal of FP64 blocks, where it is never negative: it would sum to
+// 2^-2H / 12 a row.
 template <typename TY, bool ATG>
 __global__ void __launch_bounds__(kFT, 2)
     k_sums_fix(const TY* __restrict__ Y, int ldy, int n, int s, int r, uint64_t key,
                const uint64_t* __restrict__ keyp, const int* __restrict__ ex,
                const int* __restrict__ bad, int rows_slot, int nslots, int RS, int chunk,
-               double* __restrict__ part) {
+               int shift, double* __restrict__ part) {
   if (*bad) return;
   if constexpr (ATG)
     if (keyp) key = *keyp;
+  constexpr bool kExact = !ATG && std::is_same<TY, double>::value;
   extern __shared__ __align__(16) unsigned char smem_df[];
   const int s4 = (s + 3) / 4, r4 = (r + 3) / 4, SP = 4 * s4, GP = 4 * r4;
   const int nt = ATG ? s4 * r4 : s4 * (s4 + 1) / 2;
@@ -266,26 +296,31 @@ __global__ void __launch_bounds__(kFT, 2)
         copy_async(dst + w.r * SP + w.i, src + (size_t)w.r * ldy + w.i);
     };
     long long hh[16], all[4] = {0, 0, 0, 0};
-    float cr[16];
+    float cr[16], sq[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int v = 0; v < 16; ++v) {
       hh[v] = 0;
       cr[v] = 0.f;
       T[v * kFT + threadIdx.x] = 0;
     }
-    auto fold = [&]() {
+    // half: 0 (the remainder is kept), or at a slot's end half a unit.
+    auto fold = [&](long long half) {
+      const long long mask = (1LL << shift) - 1;
 #pragma unroll
       for (int v = 0; v < 16; ++v) {
         const long long S = ATG ? (long long)((unsigned long long)all[v >> 2] - 2ULL * (unsigned long long)hh[v])
                                 : hh[v] + __float2ll_rn(cr[v] * 0x1p-32f);
-        T[v * kFT + threadIdx.x] += (S + 128) >> 8;
-        hh[v] = 0;
+        T[v * kFT + threadIdx.x] += (S + half) >> shift;
+        // A^T G: the remainder as all - 2 hh again, all its parity (that of every
+        // S of the column).
+        hh[v] = ATG ? ((all[v >> 2] & mask & 1) - (S & mask)) >> 1 : S & mask;
         cr[v] = 0.f;
       }
-      all[0] = all[1] = all[2] = all[3] = 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) all[q] &= mask & 1;
     };
     const int per = (chunk + RS - 1) / RS;  // rows of a chunk a thread takes
-    int cnt = 0, cur = 0;
+    int cnt = 0, cur = 0, it = 0;
     stage(row0, buf);
     for (int c0 = row0; c0 < row1; c0 += chunk, cur ^= 1) {
       const int rows = min(chunk, row1 - c0);
@@ -300,7 +335,7 @@ __global__ void __launch_bounds__(kFT, 2)
           const long long X = (long long)to_fixed<kAtgBits>(x, se[w.i], m);
           *reinterpret_cast<long long*>(p) = (X ^ (long long)m) - m;
         } else {
-          *p = to_limbs<kSumBits>(x, se[w.i]);
+          *p = to_limbs<Gram<TY>::kBits>(x, se[w.i]);
         }
       }
       if constexpr (ATG)
@@ -309,8 +344,8 @@ __global__ void __launch_bounds__(kFT, 2)
       __syncthreads();  // the chunk is converted; the other buffer's readers are done
       if (c0 + chunk < row1) stage(c0 + chunk, buf + (size_t)(cur ^ 1) * chunk * SP);
       if (live) {
-        if (cnt + per > kFoldRows) {
-          fold();
+        if (cnt + per > (ATG ? kAtgFold : Gram<TY>::kFold)) {
+          fold(0);
           cnt = 0;
         }
         cnt += per;
@@ -351,11 +386,31 @@ __global__ void __launch_bounds__(kFT, 2)
               cr[v] = fmaf(af[v >> 2], bl[v & 3], cr[v]);
               cr[v] = fmaf(al[v >> 2], bf[v & 3], cr[v]);
             }
+            if constexpr (kExact) {
+              if (ti == tj) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) sq[q] = fmaf(al[q], bl[q], sq[q]);
+              }
+              if (++it == Gram<TY>::kCross) {
+                it = 0;
+#pragma unroll
+                for (int v = 0; v < 16; ++v) {
+                  hh[v] += __float2int_rn(cr[v] * 0x1p-32f);
+                  cr[v] = 0.f;
+                }
+              }
+            }
           }
         }
       }
     }
-    if (live) fold();
+    if (live) {
+      if constexpr (kExact) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) hh[5 * q] += __float2ll_rn(sq[q] * 0x1p-64f);
+      }
+      fold(shift ? 1LL << (shift - 1) : 0);
+    }
     __syncthreads();
     for (int e = threadIdx.x; e < 16 * nt; e += kFT) {
       const int v = e / nt, q = e - v * nt;
@@ -371,7 +426,7 @@ __global__ void __launch_bounds__(kFT, 2)
       long long a = 0;
       for (int z = 0; z < RS; ++z) a += T[v * kFT + z * nt + q];
       const int pair = ATG ? i * r + j : i * s - i * (i - 1) / 2 + (j - i);
-      const int f = 8 + (ATG ? se[i] - kAtgBits - 32 : se[i] + se[j] - 2 * kSumBits);
+      const int f = shift + (ATG ? se[i] - kAtgBits - 32 : se[i] + se[j] - 2 * Gram<TY>::kBits);
       part[(size_t)pair * nslots + slot] = scaled(a, f);
     }
     __syncthreads();
@@ -383,7 +438,11 @@ __global__ void __launch_bounds__(kFT, 2)
 // bank conflicts), so that four loads feed 16 products.  Staged by column,
 // copied one chunk ahead, converted in place.  The factor's columns are scaled
 // so that their absolute sums (times the block's scales) stay below one, which
-// bounds the sum: |sum yh rh| <= 2^60.  The warps'
+// bounds sum |yh rh| by 2^60 and sum |yl rh| by 2^60; |yh rl| is below 2^59, so
+// the cross terms are folded every eighth product.  All three products of the
+// limbs are integer ones: with FP32 cross terms, whose sum over i is as large as
+// the result's own 24 leading bits, the columns of an orthogonalised 4,883 x 64
+// block were off by 6.9e-16 of their norm (FP64 kernels 0.9e-16).  The warps'
 // triangular loops differ in length: the columns rotate over the warps from
 // CTA to CTA, so that an SM's sub-partitions are loaded alike.
 template <bool PROJ>
@@ -425,7 +484,12 @@ __global__ void __launch_bounds__(512, 1)
     __syncthreads();
     for (int e = threadIdx.x; e < s * rc; e += blockDim.x) {
       const int i = e / rc, l = e - i * rc;
-      rt[e] = l < r ? to_limbs<kAppBits>(rd[i * r + l], ke[l] - se[i]) : make_int2(0, 0);
+      int2 a = make_int2(0, 0);
+      if (l < r) {
+        a = to_limbs30(rd[i * r + l], ke[l] - se[i]);
+        if (a.y >= 1 << 29) ++a.x, a.y -= 1 << 30;  // (|rl| <= 2^29)
+      }
+      rt[e] = a;
     }
     __syncthreads();
   }
@@ -447,38 +511,32 @@ __global__ void __launch_bounds__(512, 1)
     copy_wait();
     for (Walk w(s); w.r < rows; w.next()) {
       int2* p = b + w.i * kAppStride + w.r;
-      *p = to_limbs<kAppBits>(*reinterpret_cast<const double*>(p), se[w.i]);
+      *p = to_limbs30(*reinterpret_cast<const double*>(p), se[w.i]);
     }
     __syncthreads();
     if (n - c0 > step) stage(c0 + step, buf + (cur ^ 1) * s * kAppStride);
-    long long hh[16];
-    float cr[16];
+    long long hh[16], cr[16];
 #pragma unroll
-    for (int v = 0; v < 16; ++v) {
-      hh[v] = 0;
-      cr[v] = 0.f;
-    }
+    for (int v = 0; v < 16; ++v) hh[v] = cr[v] = 0;
     const int4* py = reinterpret_cast<const int4*>(b) + lane;
     const int4* pr = reinterpret_cast<const int4*>(rt + 4 * lt);
 #pragma unroll 2
     for (int i = 0; i < imax; ++i, py += kAppStride / 2, pr += rc / 2) {
       const int4 y0 = py[0], y1 = py[kAppRows / 4], r0 = pr[0], r1 = pr[1];
-      const int yh[4] = {y0.x, y0.z, y1.x, y1.z}, rh[4] = {r0.x, r0.z, r1.x, r1.z};
-      const float yl[4] = {__int_as_float(y0.y), __int_as_float(y0.w), __int_as_float(y1.y),
-                           __int_as_float(y1.w)};
-      const float rl[4] = {__int_as_float(r0.y), __int_as_float(r0.w), __int_as_float(r1.y),
-                           __int_as_float(r1.w)};
-      float yf[4], rf[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        yf[q] = (float)yh[q];
-        rf[q] = (float)rh[q];
-      }
+      const int yh[4] = {y0.x, y0.z, y1.x, y1.z}, yl[4] = {y0.y, y0.w, y1.y, y1.w};
+      const int rh[4] = {r0.x, r0.z, r1.x, r1.z}, rl[4] = {r0.y, r0.w, r1.y, r1.w};
 #pragma unroll
       for (int v = 0; v < 16; ++v) {
         hh[v] += (long long)yh[v >> 2] * rh[v & 3];
-        cr[v] = fmaf(yf[v >> 2], rl[v & 3], cr[v]);
-        cr[v] = fmaf(yl[v >> 2], rf[v & 3], cr[v]);
+        cr[v] += (long long)yh[v >> 2] * rl[v & 3];
+        cr[v] += (long long)yl[v >> 2] * rh[v & 3];
+      }
+      if ((i & 7) == 7) {
+#pragma unroll
+        for (int v = 0; v < 16; ++v) {
+          hh[v] += cr[v] >> 30;
+          cr[v] &= 0x3fffffff;
+        }
       }
     }
     const bool pairs = !((uintptr_t)A & 15) && !(lda & 1);
@@ -491,7 +549,7 @@ __global__ void __launch_bounds__(512, 1)
       for (int q = 0; q < 4; ++q) {
         const int l = 4 * lt + q, k = l < r ? ke[l] : 0;
         // In units of 2^(k - 60); g = +-1 joins the integer.
-        long long V = hh[4 * u + q] + __float2ll_rn(cr[4 * u + q] * 0x1p-32f);
+        long long V = hh[4 * u + q] + ((cr[4 * u + q] + (1 << 29)) >> 30);
         if constexpr (PROJ)
           V = (long long)probe_sign(key, (uint32_t)l, (uint32_t)(c0 + row)) * (1LL << (60 - min(k, 60))) - V;
         o[q] = scaled(V, k - 60);
@@ -533,13 +591,14 @@ int sums_fix(const TY* Y, int ldy, int n, int s, int r, uint64_t key, const uint
   const int s4 = div_up(s, 4), r4 = div_up(r, 4);
   const int nt = ATG ? s4 * r4 : s4 * (s4 + 1) / 2;
   const int RS = kFT / nt, wide = 4 * (ATG ? std::max(s4, r4) : s4);
-  const int chunk = RS * std::max(1, std::min(32, 2048 / (RS * wide)));
+  const int chunk = RS * std::max(1, std::min(ATG ? 32 : std::min(32, Gram<TY>::kFold), 2048 / (RS * wide)));
   const size_t smem = 16 * kFT * 8 + 2 * (size_t)chunk * 4 * s4 * 8 + (ATG ? 2 * (size_t)chunk * 4 * r4 * 4 : 0);
   auto kern = k_sums_fix<TY, ATG>;
   LD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSumsSmem));
   const int nslots = densefix_slots(n);
   kern<<<std::min(nslots, resident(kern, kFT, smem)), kFT, smem, st>>>(
-      Y, ldy, n, s, r, key, keyp, c.exp, c.bad, slot_rows(n), nslots, RS, chunk, part);
+      Y, ldy, n, s, r, key, keyp, c.exp, c.bad, slot_rows(n), nslots, RS, chunk,
+      fold_shift(slot_rows(n), ATG ? kAtgBits + 32 : 2 * Gram<TY>::kBits), part);
   LD_CHECK_LAUNCH();
   return LOGDET_OK;
 }

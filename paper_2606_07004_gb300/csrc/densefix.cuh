@@ -15,8 +15,8 @@ int densefix_slots(int n);
 
 // Per-column exponents f (|x| < 2^f) of a block, and the flag that sends the
 // products to the FP64 (or compensated FP32) kernels instead: set where a
-// column is not finite, or its largest entry is above 64 times its mean
-// magnitude.
+// column is not finite, or 2^f is above 16 times (FP32 blocks: 64 times) its
+// mean magnitude.
 struct ColScales {
   int* exp = nullptr;  // [s]
   int* bad = nullptr;  // [1]
