@@ -281,7 +281,7 @@ static int orth_t(int n, int s, const TY* Y, int ldy, TY* A, int lda, double* ws
   double* part = ws;
   double* C = part + (size_t)npairs * ntiles;
   double* Rinv = C + (size_t)s * s;
-  const bool fix = densefix_ok(n, s, std::is_same<TY, float>::value);
+  const bool fix = densefix_orth_ok(n, s, std::is_same<TY, float>::value);
   ColScales cs;
   int* keep = keep_dev;
   int* keep_tmp = nullptr;

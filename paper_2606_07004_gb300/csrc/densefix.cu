@@ -621,6 +621,19 @@ bool densefix_ok(int n, int s, bool fp32) {
   return s > 0 && (double)n * s * s >= (fp32 ? 2e8 : 2e7);
 }
 
+// Whole orthogonalisations, us, FP64 kernels / these, by n s^2: s = 7, 1e7
+// 167/161, 2e7 222/199; 20, 1e7 155/179, 2e7 216/197, 4e7 285/244; 32, 2e7
+// 239/234, 4e7 347/257; 40, 2e7 264/291, 3e7 279/295, 4e7 367/323; 50, 3e7
+// 370/386, 4e7 390/390, 6e7 535/433; 64, 4e7 526/563, 6e7 597/565 (wide blocks
+// have few slots of many column pairs).  FP32: s = 7, 1e8 526/368; 20, 1e8
+// 227/248, 2e8 352/353, 4e8 679/610; 32, 4e8 622/585; 40, 4e8 574/586, 8e8
+// 1043/953; 50, 8e8 972/1055, 1.6e9 1717/1792 (of 256 threads 182 have a tile).
+bool densefix_orth_ok(int n, int s, bool fp32) {
+  if (!densefix_ok(n, s, fp32)) return false;
+  const double w = (double)n * s * s;
+  return fp32 ? s <= 48 && w >= 4e7 * s - 1.08e9 : w >= 1e6 * s - 1.2e7;
+}
+
 size_t densefix_workspace_doubles(int s) { return (size_t)s * 4 * sm_count() + kMaxSketch + 2; }
 
 int densefix_slots(int n) { return div_up(n, slot_rows(n)); }

@@ -5,9 +5,11 @@
 
 namespace ld {
 
-// Whether a block of n rows and s columns takes the fixed-point products (FP32
-// blocks from a larger size).
+// Whether the projection of a block of n rows and s columns takes the
+// fixed-point products (FP32 blocks from a larger size), and whether its
+// orthogonalisation does (a part of those).
 bool densefix_ok(int n, int s, bool fp32 = false);
+bool densefix_orth_ok(int n, int s, bool fp32);
 // Workspace (doubles) of column_scales for s columns.
 size_t densefix_workspace_doubles(int s);
 // Partial slots of gram_fix and atg_fix: at most one per 256 rows.

@@ -63,3 +63,23 @@ def test_orthonormal_columns_over_the_accepted_range(n, s, rho):
     print(f"n {n} s {s} rho {rho}: norms {off:.1e}, columns {err:.1e} rms {rms:.1e}")
     assert off <= 1e-15
     assert err <= 4e-16
+
+
+@pytest.mark.parametrize("dtype,few,many", [
+    # Where the FP64 (compensated FP32) kernels are faster, and where these are.
+    (torch.float64, (4883, 64), (13007, 64)), (torch.float64, (9001, 50), (16001, 50)),
+    (torch.float64, (40001, 20), (50021, 20)), (torch.float32, (400001, 50), (600001, 40)),
+    (torch.float32, (300001, 24), (400001, 24))])
+def test_which_products_a_block_takes(dtype, few, many):
+    # The fixed-point products launch four kernels more a round (three for FP32).
+    orth = B.logdet_orth if dtype == torch.float64 else B.logdet_orth_f32
+
+    def launches(n, s):
+        y = torch.randn(n, s, dtype=dtype, device="cuda")
+        a = torch.empty_like(y)
+        before = B.logdet_launch_count()
+        orth(n, s, y, s, a, s)
+        return B.logdet_launch_count() - before
+    small = launches(1001, few[1])
+    assert launches(*few) == small
+    assert launches(*many) == small + (8 if dtype == torch.float64 else 6)
