@@ -195,6 +195,14 @@ int logdet_grid_structure(logdet_handle h, int32_t* dim, int32_t* line_stride, i
 int logdet_grid_structure_csr(int32_t n, const int32_t* rowptr, const int32_t* colind,
                               int32_t* dim, int32_t* line_stride, int32_t* reach);
 
+/* How the estimators apply a gridded operator to blocks whose narrowest has
+ * `columns` columns, in `precision` (LOGDET_FP64 or LOGDET_MIXED_FP32):
+ * *log2_x = *log2_y = *windows = 0 directly, otherwise by Fourier transforms of
+ * 2^log2_x by 2^log2_y points over *windows windows of the grid.  Errors: EINVAL
+ * (null pointer, a CSR handle, columns < 1, another precision). */
+int logdet_grid_transform(logdet_handle h, int32_t precision, int32_t columns, int32_t* log2_x,
+                          int32_t* log2_y, int32_t* windows);
+
 /* ---- estimators --------------------------------------------------------
  * logdet_oslq: Algorithm 3 (OSLQ, Sec. 3): J = Q/alpha with alpha the upper
  * spectral bound; s = floor(num_probes/3) Rademacher sketch columns give

@@ -35,7 +35,7 @@ ST_BREAKDOWN, ST_NONPOS_RITZ, ST_RANK_DEFICIENT, ST_LOG_FAILED = 1, 2, 4, 8
 EXPORTED = [
     "logdet_opts_default", "logdet_strerror", "logdet_last_error",
     "logdet_create", "logdet_create_device", "logdet_create_grid", "logdet_destroy", "logdet_info",
-    "logdet_grid_structure", "logdet_grid_structure_csr", "logdet_oslq", "logdet_osaiop",
+    "logdet_grid_structure", "logdet_grid_structure_csr", "logdet_grid_transform", "logdet_oslq", "logdet_osaiop",
     "logdet_probe_fill", "logdet_probe_fill_gaussian", "logdet_spmm", "logdet_quadform",
     "logdet_orth", "logdet_orth_f32",
     "logdet_gauss_quadrature_log", "logdet_hessenberg_log_e1",
@@ -104,6 +104,8 @@ _sig("logdet_create_grid", C.c_int, [_i32, _i32, _i32, _P, C.POINTER(_P)])
 _sig("logdet_destroy", None, [_P])
 _sig("logdet_info", C.c_int, [_P, C.POINTER(_i32), C.POINTER(_i64), C.POINTER(_dbl), C.POINTER(_dbl)])
 _sig("logdet_grid_structure", C.c_int, [_P, C.POINTER(_i32), C.POINTER(_i32), C.POINTER(_i32)])
+_sig("logdet_grid_transform", C.c_int, [_P, _i32, _i32, C.POINTER(_i32), C.POINTER(_i32),
+                                        C.POINTER(_i32)])
 _sig("logdet_grid_structure_csr", C.c_int, [_i32, _P, _P, C.POINTER(_i32), C.POINTER(_i32),
                                             C.POINTER(_i32)])
 for _n in ("logdet_oslq", "logdet_osaiop"):
@@ -316,6 +318,15 @@ class Handle:
         _check(_lib.logdet_grid_structure(self._h, C.byref(dim), C.byref(L), C.byref(A)),
                "logdet_grid_structure")
         return dim.value, L.value, A.value
+
+    def grid_transform(self, precision, columns):
+        """(log2 of x points, log2 of y points, windows) of the Fourier
+        transforms that apply a gridded operator to blocks of `columns`
+        columns, (0, 0, 0) when it is applied directly (logdet_grid_transform)."""
+        lx, ly, w = _i32(), _i32(), _i32()
+        _check(_lib.logdet_grid_transform(self._h, precision, columns, C.byref(lx), C.byref(ly),
+                                          C.byref(w)), "logdet_grid_transform")
+        return lx.value, ly.value, w.value
 
     def _run(self, fn, name, num_probes, krylov_steps, iop_window, seed, precision, tol,
              lam, stream, shift=0.0, autotune=0, plain=0, gaussian=0, block_width=0):

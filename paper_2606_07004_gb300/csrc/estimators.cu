@@ -178,6 +178,21 @@ int logdet_grid_structure_csr(int32_t n, const int32_t* rowptr, const int32_t* c
   return LOGDET_OK;
 }
 
+int logdet_grid_transform(logdet_handle h, int32_t precision, int32_t columns, int32_t* log2_x,
+                          int32_t* log2_y, int32_t* windows) {
+  if (!h || h->kind != 1 || !log2_x || !log2_y || !windows || columns < 1 || columns > 1 << 20 ||
+      (precision != LOGDET_FP64 && precision != LOGDET_MIXED_FP32)) {
+    set_error("grid transform: NULL pointer, CSR handle or argument out of range");
+    return LOGDET_EINVAL;
+  }
+  const int ld = round_up(columns, precision_vec(precision));
+  const GridFft f = precision == LOGDET_FP64 ? grid_fft_plan<double>(h, ld) : grid_fft_plan<float>(h, ld);
+  *log2_x = f.pairs ? f.lnx : 0;
+  *log2_y = f.pairs ? f.lny : 0;
+  *windows = f.pairs ? f.tx * f.ty : 0;
+  return LOGDET_OK;
+}
+
 int logdet_oslq(logdet_handle h, int32_t P, int32_t m, int32_t k, uint64_t seed,
                 const logdet_opts* opts, logdet_result* out) {
   return run_estimator(0, h, P, m, k, seed, opts, out);
