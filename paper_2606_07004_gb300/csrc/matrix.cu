@@ -4,6 +4,7 @@
 #include "dia.cuh"
 #include "krylov.cuh"
 #include "profile.cuh"
+#include "quotient.cuh"
 
 #include <atomic>
 #include <cmath>
@@ -394,34 +395,25 @@ void destroy_handle(logdet_ctx* h) {
 }
 
 // Scaled copy of the values: out[i] = (T)(vals[i] / c), the division in FP64.
-// For FP32 results the quotient comes from the reciprocal y = 1 / c and one
-// residual correction (Markstein, IBM J. Res. Dev. 34, 1990), within 2^-52 of
-// half a unit of FP64: three FP64 operations, where the division bounded the
-// pass (28M values: 450 -> 268 us, 50 at the memory's rate; the grid stencils'
-// values by diagonal copy these instead of dividing again: 448 -> 141 us).
+// For FP32 results the quotient comes from the reciprocal y = 1 / c
+// (quotient.cuh): the division bounded the pass (28M values: 450 -> 268 us, 50 at
+// the memory's rate; the grid stencils' values by diagonal copy these instead of
+// dividing again: 448 -> 141 us).
 template <typename Vin, typename T>
 __global__ void k_scale_vals(const Vin* __restrict__ in, long long nnz, double c, double y,
                              T* __restrict__ out) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nnz;
        i += (long long)gridDim.x * blockDim.x) {
     const double a = (double)in[i];
-    if constexpr (std::is_same<T, float>::value) {
-      // (zero, and exponents where the residual could leave the range)
-      const int e = (__double2hiint(a) >> 20) & 0x7ff;
-      if (y != 0.0 && e > 1023 - 400 && e < 1023 + 400) {
-        const double q = a * y;
-        out[i] = (T)fma(fma(-q, c, a), y, q);
-        continue;
-      }
-    }
-    out[i] = (T)(a / c);
+    if constexpr (std::is_same<T, float>::value) out[i] = scaled_quotient(a, c, y);
+    else out[i] = (T)(a / c);
   }
 }
 
 template <typename T>
 int scaled_values(logdet_ctx* h, double c, T* out, cudaStream_t st) {
   const int blocks = 8 * sm_count();
-  const double y = std::fabs(c) > 1e-100 && std::fabs(c) < 1e100 ? 1.0 / c : 0.0;
+  const double y = quotient_reciprocal(c);
   ProfScope prof(KC_OTHER, st);
   if (h->vals_dtype == LOGDET_VALS_F64)
     k_scale_vals<double, T><<<blocks, 256, 0, st>>>((const double*)h->vals, h->nnz, c, y, out);
