@@ -1,7 +1,7 @@
 // FP64 SpMM pass of grid stencil matrices in fixed point.
 //
-// An FP64 instruction takes a sub-partition 64 clocks on this GPU, a 32 x 32
-// + 64-bit integer multiply-add two, so the product y = A x of an FP64 block
+// An FP64 instruction takes a sub-partition 64 clocks and more on this GPU (78
+// measured), a 32 x 32 + 64-bit integer multiply-add 4.7, so the product y = A x of an FP64 block
 // is summed in integers.  Each column of x becomes X = x 2^60 / F (truncated
 // to an integer below 2^60), F a power of two 32 to 128 times the column's
 // root mean square (from sigma, which is 1 / |u|), and each matrix entry
@@ -15,8 +15,12 @@
 // stays below 2^63 for up to 13 entries (longer rows fold it every eight).
 // The result is rounded to FP64 once.  Its error, a few units of 2^-60 F, is
 // below that of an FP64 sum, which rounds every product and addition to 2^-53
-// of its size; measured against 64-bit references the estimates' errors are
-// unchanged (3e-16 to 1e-15).  An entry of x too large for its column's F (or not finite) sets
+// of its size.  (x and the entries are cut at 2^-60 of F and of the largest row
+// sum, so a number far below those keeps fewer bits than FP64's 53; a product's
+// error is measured by the norms, as the recurrences use it.)  Quadratic forms of
+// 12 Lanczos steps against extended precision, 120 probes each, rms error here /
+// of the CSR pass: 3D Laplacian 1.25e-15 / 1.02e-15, 2D 0.90e-15 / 1.44e-15,
+// Matern 0.29e-15 / 0.52e-15.  An entry of x too large for its column's F (or not finite) sets
 // the job's flag; k_spmm_fix_general, launched after every product, then redoes
 // it with FP64 arithmetic, and takes the job's later products alone.
 //

@@ -9,7 +9,11 @@ namespace ld {
 
 // Blocks smaller than this keep the CSR pass: their steps are bound by the
 // latency of dependent launches, not by the FP64 pipe (a 64 x 64 grid's pass
-// takes 4 us of which the pipe is busy 0.8).
+// takes 4 us of which the pipe is busy 0.8).  Solves of 20 steps, us, CSR pass /
+// this one, by the MB of the narrower block: 3D Laplacian OSLQ 4 MB 1184/1451,
+// 8 2012/1826, 16 3445/2485, 34 5199/4191; OSA-IOP window 4 8 4246/4164, 16
+// 7357/5785; 2D Laplacian window 4 8 3904/3992, 16 6644/5899; Matern OSLQ 8
+// 2703/2421, window 4 8 5266/5899, 16 9493/7440.
 constexpr size_t kFixMinBlock = (size_t)16 << 20;
 
 // Geometry of a slice of `width` columns of an FP64 block; false when the matrix has no
