@@ -763,9 +763,11 @@ __global__ void __launch_bounds__(512, update_min_ctas<T, NB>())
 constexpr int kRedLanes = 4;  // independent accumulators per thread
 // Up to this many partials per dot the scalar steps run one warp per dot in a
 // CTA per probe (k_scalar_small): 64 x 64 grid, FP64, 256 partials: 13.4 us a
-// launch in the counter form's code, 6.6 us so; a warp per dot over the 4096
-// partials of a 2M-row block would read 128 of them one wave after another.
-constexpr int kSmallTiles = 1024;
+// launch in the counter form's code, 6.6 us so.  With more a warp reads them one
+// wave after another: FP64 solves of 30 steps, us, one warp per dot / k_scalar,
+// 506 partials 792/730 (window 4 1754/1619), 512 2647/2446 (window 4), 341
+// 1202/1142; FP32 640/606, 739/691, 1075/1000.
+constexpr int kSmallTiles = 256;
 
 
 // Sum of the ntiles partials of (dot d, column p) by a CTA of kRedThreads
@@ -1421,6 +1423,9 @@ static void launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t sme
   cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// Blocks (of all jobs) up to this size: pass 1 overlaps the launch before it.
+constexpr size_t kOverlapMaxBytes = (size_t)16 << 20;
+
 template <typename T>
 int launch_spmm(const SpmmBatch<T>& b, int threads, cudaStream_t s) {
   int nd = 0;
@@ -1432,9 +1437,11 @@ int launch_spmm(const SpmmBatch<T>& b, int threads, cudaStream_t s) {
   using Acc = typename AccOf<T>::type;
   size_t smem = (size_t)threads * Vec16<T>::N * sizeof(Acc);
   double flops = 0.0, bytes = 0.0;
+  size_t block_bytes = 0;
   for (int j = 0; j < b.njobs; ++j) {
     const SpmmJob<T>& J = b.jobs[j];
     const double vb = (double)J.n * J.b * sizeof(T);
+    block_bytes += (size_t)J.n * J.width * sizeof(T);
     const int extra_reads = J.ndots - ((J.ndots > 0 && J.dotv[0] == J.x) ? 1 : 0);
     flops += 2.0 * (double)J.nnz * J.b + 2.0 * (double)J.n * J.b * J.ndots;
     bytes += 4.0 * (J.n + 1) + (double)J.nnz * (4 + sizeof(typename ValOf<T>::type)) +
@@ -1445,13 +1452,18 @@ int launch_spmm(const SpmmBatch<T>& b, int threads, cudaStream_t s) {
   {                                                                           \
     auto kern = items ? spmm_kernel<T, ND, true>() : spmm_kernel<T, ND, false>(); \
     int grid = persistent_grid(kern, threads, smem, b.total_tiles);           \
-    if (b.total_tiles <= kSmallTiles) launch_pdl(kern, dim3(grid), dim3(threads), smem, s, b); \
+    if (overlap) launch_pdl(kern, dim3(grid), dim3(threads), smem, s, b);     \
     else kern<<<grid, threads, smem, s>>>(b);                                 \
     break;                                                                    \
   }
   // A large pass 1 is launched without the overlap: it follows the update
   // pass, and CTAs resident beside that pass's ran 4 % slower (128^3 FP64,
-  // window 4: 211.4 ms a solve against 206.0).
+  // window 4: 211.4 ms a solve against 206.0).  2D Laplacian, 20 columns, 30
+  // steps, us, with / without: FP64 10 MB 1619/1694 (window 4 4049/4055), 21 MB
+  // 2674/2739 (6537/6574), 42 MB 4633/4621 (11288/11353), 84 MB 9291/9007
+  // (22027/21443); FP32 5 MB 1099/1156 (2882/2944), 10 MB 1386/1438 (3814/3782),
+  // 21 MB 2277/2283 (6140/6004).
+  const bool overlap = block_bytes <= kOverlapMaxBytes;
   do {
     if (nd == 0) LD_SPMM_CASE(0)
     if (nd == 1) LD_SPMM_CASE(1)
