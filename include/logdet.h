@@ -47,7 +47,10 @@ extern "C" {
 #define LOGDET_VALS_F64  0
 #define LOGDET_VALS_F32  1
 
-#define LOGDET_FP64        0  /* everything in IEEE binary64 */
+#define LOGDET_FP64        0  /* IEEE binary64 throughout; the products of large grid
+                                 stencils and of the Hutch++ split of large blocks are
+                                 summed in 60-bit fixed point (no less exact than
+                                 binary64 sums, measured by the norms) and rounded once */
 #define LOGDET_MIXED_FP32  1  /* FP32 values and vectors, compensated FP32 dots,
                                  OSLQ's Hutch++ QR and projection in FP32 with
                                  compensated Gram sums (FP64 Cholesky factor),
@@ -176,8 +179,8 @@ void logdet_destroy(logdet_handle h);
 int logdet_info(logdet_handle h, int32_t* n, int64_t* nnz, double* gersh_lo, double* gersh_hi);
 
 /* Grid structure found at creation from host CSR arrays (n >= 4096), which
- * mixed-FP32 solves use to run the SpMM pass as a sweep over TMA-staged
- * windows of x instead of CSR gathers.  *dim = 2: every entry on one of at
+ * mixed-FP32 solves, and FP64 solves whose blocks are above 16 MB, use to run
+ * the SpMM pass as a sweep over TMA-staged windows of x instead of CSR gathers.  *dim = 2: every entry on one of at
  * most 16 diagonals with offsets l * L + c, |l| <= *reach <= 3, c within a
  * range of at most 16 (a 2D grid stencil, L the grid's row length): a line
  * sweep.  *dim = 3: a stencil on an L x ny x nz grid (row (z ny + y) L + x)
@@ -305,8 +308,9 @@ int logdet_orth(int32_t n, int32_t s, const double* y_dev, int32_t ldy, double* 
 
 /* logdet_orth_f32: the same step for an FP32 block, as mixed-precision OSLQ
  * runs it (Algorithm 3's QR of Y = J S): two rounds of Cholesky QR whose Gram
- * sums are compensated FP32 dots (Dot2) accumulated per 256-row tile and
- * summed in FP64, an FP64 Cholesky factor, and FP32 applies of its inverse.
+ * sums are compensated FP32 dots (Dot2) accumulated per tile of at most 256
+ * rows, or fixed-point sums for large blocks, summed in FP64, an FP64 Cholesky
+ * factor, and FP32 applies of its inverse.
  * A (FP32, n x s in a block of leading dimension lda, a_dev may alias y_dev)
  * is orthonormal to FP32 rounding and spans the FP32 Y's columns; the column
  * drop rule and *s_eff are those of logdet_orth.  Products y_i y_j are formed
