@@ -889,6 +889,19 @@ struct Solve : ISolve {
                               st, tc);
   }
 
+  // A Krylov run that applies this solve's operator: the scaled values, or the
+  // tables and the cover that belong to them.
+  void new_run() {
+    run.reset(new KRun<T>(st));
+    run->colshift = cshift.p;
+    run->hctx = h;
+    run->gtab = gtabs.p;
+    run->gfft = gfft;
+    run->diavals = diav.p;
+    run->fixvals = fixv.p;
+    run->fix_ka = fix_ka;
+  }
+
   // Start the Krylov run of the current phase on X0 (a group member only
   // records it for the group).
   int start_run(int b_, int ld_, int k_, int method_, bool track_e_, T* X0, T* Vfull, TuneCfg tc) {
@@ -1011,20 +1024,13 @@ struct Solve : ISolve {
       LD_TRY(cshift.alloc(cnt));
       LD_TRY(fill_double(cshift.p, cnt, c.shift / cscale, st));
     }
-    run.reset(new KRun<T>(st));
+    new_run();
     if (s == 0) {
       // Plain SLQ: no sketch; the residual probes are the probes themselves.
       LD_TRY(hutchpp_split(n, 0, r, nullptr, lds, probe_key(c.seed, 1), X64, ld, keep.p, st,
                            c.gaussian, dkey(1)));
       T* X0;
       LD_TRY(make_x0(&X0));
-      run->colshift = cshift.p;
-      run->hctx = h;
-      run->gtab = gtabs.p;
-      run->gfft = gfft;
-      run->diavals = diav.p;
-      run->fixvals = fixv.p;
-      run->fix_ka = fix_ka;
       TuneCfg tc;
       LD_TRY(layout(ld, c.method == 1, &tc));
       if (c.method == 0) {
@@ -1071,13 +1077,6 @@ struct Solve : ISolve {
                              dkey(1)));
         LD_TRY(make_x0(&X0));
       }
-      run->colshift = cshift.p;
-      run->hctx = h;
-      run->gtab = gtabs.p;
-      run->gfft = gfft;
-      run->diavals = diav.p;
-      run->fixvals = fixv.p;
-      run->fix_ka = fix_ka;
       TuneCfg tc;
       LD_TRY(layout(ld, false, &tc));
       LD_TRY(start_run(b, ld, 2, 0, false, X0, nullptr, tc));
@@ -1086,13 +1085,6 @@ struct Solve : ISolve {
       // (a group member fills only the start block; the group keeps the basis)
       LD_TRY(Vst.alloc((size_t)n * lds * (grouped ? 1 : m)));
       LD_TRY(probe_fill<T>(probe_key(c.seed, 0), n, s, 0, Vst.p, lds, st, c.gaussian, dkey(0)));
-      run->colshift = cshift.p;
-      run->hctx = h;
-      run->gtab = gtabs.p;
-      run->gfft = gfft;
-      run->diavals = diav.p;
-      run->fixvals = fixv.p;
-      run->fix_ka = fix_ka;
       TuneCfg tc;
       LD_TRY(layout(lds, false, &tc));
       LD_TRY(start_run(s, lds, kk, 1, false, Vst.p, Vst.p, tc));
@@ -1143,14 +1135,7 @@ struct Solve : ISolve {
     Y64.release();
     T* X0;
     LD_TRY(make_x0(&X0));
-    run.reset(new KRun<T>(st));
-    run->colshift = cshift.p;
-    run->hctx = h;
-    run->gtab = gtabs.p;
-    run->gfft = gfft;
-    run->diavals = diav.p;
-    run->fixvals = fixv.p;
-    run->fix_ka = fix_ka;
+    new_run();
     TuneCfg tc;
     LD_TRY(layout(ld, true, &tc));
     LD_TRY(start_run(b, ld, kk, 1, true, X0, nullptr, tc));
