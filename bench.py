@@ -1021,7 +1021,7 @@ def small2d_case(args):
         t_b = time.perf_counter() - t0
         launches_b = (B.logdet_launch_count() - c0) / N
         # the same blocking solves with the Krylov phase as one persistent
-        # launch (opt-in) instead of four launches per step
+        # launch (opt-in) instead of three launches per step
         os.environ["LOGDET_KRYLOV_PERSISTENT"] = "1"
         h.oslq(P, m, seed=0)
         c0 = B.logdet_launch_count()
@@ -1076,7 +1076,7 @@ def small2d_case(args):
         "workload": "2D Laplacian 64^2 + 0.1 I (n=4096, nnz=%d), OSLQ m=30, 30 probes, FP64" % A.nnz,
         "metric": METRIC, "unit": UNIT, "dtype": "f64",
         "blocking": {"value": N / t_b, "latency_ms": {"p50": _pct(lat_b, 0.5), "p99": _pct(lat_b, 0.99)},
-                     "launches_per_solve": launches_b, "krylov": "four launches per step"},
+                     "launches_per_solve": launches_b, "krylov": "three launches per step"},
         "blocking_persistent": {"value": N / t_s_b,
                                 "latency_ms": {"p50": _pct(lat_s, 0.5), "p99": _pct(lat_s, 0.99)},
                                 "launches_per_solve": launches_s,
