@@ -65,6 +65,24 @@ def test_orthonormal_columns_over_the_accepted_range(n, s, rho):
     assert err <= 4e-16
 
 
+@pytest.mark.parametrize("n,s", [(50021, 20), (20011, 32)])
+@pytest.mark.parametrize("kappa", [1e1, 1e3, 1e5])
+def test_correlated_columns(n, s, kappa):
+    # Columns of condition kappa, as a sketch's are: the applies' sums cancel, and
+    # what an entry of Y or of the inverse factor loses counts kappa times.  The
+    # FP64 kernels are off by 1.2e-17 to 3.1e-17 kappa there.
+    rng = np.random.default_rng(7)
+    u, v = (np.linalg.qr(rng.standard_normal((s, s)))[0] for _ in range(2))
+    y = rng.standard_normal((n, s)) @ (u * np.logspace(0, -np.log10(kappa), s)) @ v
+    yd = torch.as_tensor(y, device="cuda")
+    a = torch.empty_like(yd)
+    assert B.logdet_orth(n, s, yd, s, a, s) == s
+    a = a.cpu().numpy()
+    g = np.einsum("ni,nj->ij", a.astype(np.longdouble), a.astype(np.longdouble))
+    assert np.abs(g - np.eye(s)).max() <= 1e-15
+    assert np.sqrt(((a - _qr(y)) ** 2).sum(0)).max() <= 4e-16 + 3e-17 * kappa
+
+
 @pytest.mark.parametrize("dtype,few,many", [
     # Where the FP64 (compensated FP32) kernels are faster, and where these are.
     (torch.float64, (4883, 64), (13007, 64)), (torch.float64, (9001, 50), (16001, 50)),
